@@ -186,8 +186,12 @@ int make_box(const nf_box& in, bool need_force, BoxDev* out)
         }
     }
     const double w = in.box / in.K;
-    b.scale_acc = 1.0 / ((double)in.N * w * w);
-    b.scale_grad = 1.0 / ((double)in.N * w * w * w);
+    const double scale_acc = 1.0 / ((double)in.N * w * w), scale_grad = 1.0 / ((double)in.N * w * w * w);
+    b.mass = 1.0 / (double)in.N;
+    b.acc_hi = (float)scale_acc;
+    b.acc_lo = (float)(scale_acc - (double)b.acc_hi);
+    b.grad_hi = (float)scale_grad;
+    b.grad_lo = (float)(scale_grad - (double)b.grad_hi);
     if (need_force) {
         if (in.R < 1 || in.R > NF_MAX_R) return fail(NF_ERR_ARG, "R = %d out of [1, %d]", in.R, NF_MAX_R);
         if (in.K < 2 * in.R + 1)

@@ -980,14 +980,19 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e)
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
 
-__global__ void __launch_bounds__(256)
+// One particle a thread: its row of partials is one round of independent
+// loads, so a small box (64^3: 1024 blocks) is as latency-hidden as a large
+// one.  Blocks of 4096 particles took 21 us for any box below 512k particles
+// (16 rounds in a row on a few blocks); with one round the whole nf_forces
+// call of 4096 particles went from 171 to 158 us, of 32768 from 279 to 264.
+__global__ void __launch_bounds__(kCombineChunk)
 k_combine(const BoxDev* __restrict__ boxes, int nboxes, const float4* __restrict__ partial, int pstride,
           float* __restrict__ out, float* __restrict__ rho, double* __restrict__ chunk_sums, bool adjoint)
 {
-    // block = one chunk of kCombineChunk particles (original order) of a single box;
-    // a particle's 2R+1 partials are one contiguous row, so the loads and the
+    // block = one chunk of particles (original order) of a single box; a
+    // particle's 2R+1 partials are one contiguous row, so the loads and the
     // output rows of a warp are both contiguous
-    __shared__ double red[3][8];
+    __shared__ double red[3][kCombineChunk / 32];
     int chunk = blockIdx.x;
     int lo = 0, hi = nboxes - 1;
     while (lo < hi) {
@@ -997,17 +1002,14 @@ k_combine(const BoxDev* __restrict__ boxes, int nboxes, const float4* __restrict
     }
     const BoxDev& B = boxes[lo];
     const int nslot = 2 * B.R + 1;
-    const double scale = adjoint ? B.scale_grad : B.scale_acc;
     // the scale as an unevaluated float pair: scale = s_hi + s_lo to ~2^-48
-    const float s_hi = (float)scale;
-    const float s_lo = (float)(scale - (double)s_hi);
-    const double m = 1.0 / (double)B.N;
+    const float s_hi = adjoint ? B.grad_hi : B.acc_hi;
+    const float s_lo = adjoint ? B.grad_lo : B.acc_lo;
     const bool out_aligned8 = (reinterpret_cast<uintptr_t>(out) & 7) == 0;
-    const int e0 = B.part_base + (chunk - B.chunk_base) * kCombineChunk;
-    const int e1 = min(e0 + kCombineChunk, B.part_base + B.N);
+    const int e = B.part_base + (chunk - B.chunk_base) * kCombineChunk + (int)threadIdx.x;
     double net[3] = {0.0, 0.0, 0.0};
     constexpr int kMaxSlots = 2 * NF_MAX_R + 1;
-    for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
+    if (e < B.part_base + B.N) {
         const float4* row_in = partial + (size_t)e * (size_t)pstride;
         // issue every partial load first (they are independent), then sum
         float4 v[kMaxSlots];
@@ -1033,7 +1035,7 @@ k_combine(const BoxDev* __restrict__ boxes, int nboxes, const float4* __restrict
             const float perr = __fmaf_rn(sh, s_hi, -p);
             const float a = __fadd_rn(p, __fmaf_rn(sh, s_lo, __fmaf_rn(sl, s_hi, perr)));
             a3[c] = a;
-            if (chunk_sums) net[c] += m * (double)a;
+            if (chunk_sums) net[c] = B.mass * (double)a;
         }
         // the particle's row goes out in two stores (its 12 bytes start 8-byte
         // aligned for even e, 4 bytes past it for odd e)
@@ -1081,17 +1083,27 @@ k_combine(const BoxDev* __restrict__ boxes, int nboxes, const float4* __restrict
     }
 }
 
-__global__ void k_net(const BoxDev* __restrict__ boxes, int nboxes, const double* __restrict__ chunk_sums,
-                      double* __restrict__ net)
+// Net force of box blockIdx.x: its chunk sums, each thread a strided share in
+// order, then a fixed tree (the same sum for the same N in any batch).
+constexpr int kNetThreads = 256;
+__global__ void __launch_bounds__(kNetThreads)
+k_net(const BoxDev* __restrict__ boxes, const double* __restrict__ chunk_sums, double* __restrict__ net)
 {
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nboxes) return;
+    __shared__ double red[3][kNetThreads];
+    const int b = blockIdx.x, t = threadIdx.x;
     const BoxDev& B = boxes[b];
-    int n = (B.N + kCombineChunk - 1) / kCombineChunk;
+    const int n = (B.N + kCombineChunk - 1) / kCombineChunk;
     double v[3] = {0.0, 0.0, 0.0};
-    for (int q = 0; q < n; ++q)
-        for (int c = 0; c < 3; ++c) v[c] += chunk_sums[3 * (size_t)(B.chunk_base + q) + c];
-    for (int c = 0; c < 3; ++c) net[3 * (size_t)b + c] = v[c];
+    for (int q = t; q < n; q += kNetThreads)
+        for (int c = 0; c < 3; ++c) v[c] += chunk_sums[3 * ((size_t)B.chunk_base + q) + c];
+    for (int c = 0; c < 3; ++c) red[c][t] = v[c];
+    __syncthreads();
+    for (int h = kNetThreads / 2; h; h >>= 1) {
+        if (t < h)
+            for (int c = 0; c < 3; ++c) red[c][t] += red[c][t + h];
+        __syncthreads();
+    }
+    if (t < 3) net[3 * (size_t)b + t] = red[t][0];
 }
 
 int grid_for(size_t n, int threads)
@@ -1239,7 +1251,7 @@ cudaError_t launch_combine(bool adjoint, const BoxDev* boxes, int nboxes, int nc
                            int pstride, float* out, float* rho, double* chunk_sums, cudaStream_t s)
 {
     if (nchunks <= 0) return cudaSuccess;
-    k_combine<<<nchunks, 256, 0, s>>>(boxes, nboxes, partial, pstride, out, rho, chunk_sums, adjoint);
+    k_combine<<<nchunks, kCombineChunk, 0, s>>>(boxes, nboxes, partial, pstride, out, rho, chunk_sums, adjoint);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -1247,7 +1259,7 @@ cudaError_t launch_combine(bool adjoint, const BoxDev* boxes, int nboxes, int nc
 cudaError_t launch_net(const BoxDev* boxes, int nboxes, const double* chunk_sums, double* net,
                        cudaStream_t s)
 {
-    k_net<<<(nboxes + 63) / 64, 64, 0, s>>>(boxes, nboxes, chunk_sums, net);
+    k_net<<<nboxes, kNetThreads, 0, s>>>(boxes, chunk_sums, net);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -34,8 +34,11 @@ struct BoxDev {
     int N;
     int chunk_base;  // first combine chunk of this box
     double kl;       // K / box, multiplies a box-unit coordinate into cell units
-    double scale_acc;   // m / w^2: cell-unit pair sums -> box-unit acceleration
-    double scale_grad;  // m / w^3: cell-unit Jacobian sums -> box-unit gradient
+    double mass;     // m = 1 / N
+    // as unevaluated float pairs (hi, lo), to 2^-48:
+    float acc_hi, acc_lo;    // m / w^2: cell-unit pair sums -> box-unit acceleration
+    float grad_hi, grad_lo;  // m / w^3: cell-unit Jacobian sums -> box-unit gradient
+    double pad;
     // Eq. (spline) in cell units: f(r) = min(c0 + r^2 (c2 + c1 / r), 1 / r^3)
     float c0, c1, c2;
     float eps2;      // eps_s^2 (cell units^2)
@@ -82,7 +85,7 @@ struct BoxFill {
     BoxDev b[kMaxBoxesPerFill];
 };
 
-constexpr int kCombineChunk = 4096;  // particles per combine block (never straddles boxes)
+constexpr int kCombineChunk = 256;   // particles per combine block, one a thread (never straddles boxes)
 constexpr int kBuckets = 64;         // cost buckets of the LPT work order
 
 // Scratch of the time-step reduction (nf_step.cu).
