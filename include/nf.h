@@ -112,10 +112,12 @@ int nf_bin(const float *pos, int64_t N, double box, int K,
  *        (2R+1)^3 cells around i's cell (j = i included; it adds 0).
  *   net  [3] FP64 (output) or NULL: sum_i (1/N) a_i of the FP32 results,
  *        accumulated in FP64 (zero up to roundoff by Newton's third law).
- * The pair arithmetic runs in FP32 on cell-relative coordinates.  The 2R+1
- * pencil partial sums that reach each particle are added without rounding
- * error into an FP32 (hi, lo) pair (a TwoSum cascade), multiplied by the box
- * scale m/w^2 held as a float pair, and rounded once to FP32. */
+ * The pair arithmetic runs in FP32 on cell-relative coordinates.  The partial
+ * sums that reach each particle (one per pencil that it is a sink of and, in the
+ * symmetric kernel, one per half-plane cell that it is a source of) are added
+ * without rounding error into an FP32 (hi, lo) pair (a TwoSum cascade),
+ * multiplied by the box scale m/w^2 held as a float pair, and rounded once to
+ * FP32.  A call always gives the same bits for the same inputs. */
 int nf_forces(const float *pos, int64_t N, double box, int K, int R, double eps,
               float *acc, double *net, void *ws, size_t ws_bytes, void *stream);
 
@@ -190,7 +192,11 @@ typedef struct {
  *                   not for nf_forces_density, which then runs its usual
  *                   build at one block per SM).
  * Unsupported combinations are rejected with NF_ERR_ARG.  The built-in
- * defaults are below. */
+ * defaults are below.  Under the built-in tuning of a direction, boxes of 2^18
+ * to 2^28 particles run in the symmetric kernel, which meets every pair once and
+ * applies it to both particles, unless much of a box's work lies in a few dense
+ * pencils (decided on the device, per box); any other tuning, and the time
+ * steps, run the directed kernel that it shapes. */
 typedef struct {
     int sinks_per_lane;
     int stage;
@@ -416,7 +422,7 @@ int nf_timestep(const float *pos, const float *vel, const float *acc, int64_t N,
 /* One leapfrog step in place, all on the device:
  *     vel += acc dt/2;  pos = wrap(pos + vel dt) into [0, box);
  *     acc = nf_forces(pos);  vel += acc dt/2;
- * acc must hold the accelerations at the input positions (from nf_forces or
+ * (nf_forces by the directed kernel at every size, see nf_tuning.)  acc must hold the accelerations at the input positions (from nf_forces or
  * the previous step).  dt is ONE double in device memory: it is read for this
  * step and, when prm != NULL, overwritten with the next step's dt from
  * Eq. (timestep) at the new state; so a loop of steps needs no host round trip
@@ -465,7 +471,8 @@ int nf_status_read(void *ws, void *stream);
  * stream synchronisation (host array out[4]):
  *   out[0] = pair interactions computed, P = sum_c n_c S_c (self pairs
  *            included), summed over boxes;
- *   out[1] = work items (sink chunks) in the persistent queue;
+ *   out[1] = work items (sink chunks, or units of the symmetric kernel) in the
+ *            persistent queue;
  *   out[2] = largest cell occupancy;
  *   out[3] = sink lanes issued (32 * sinks_per_lane rounded up per chunk),
  *            so out[0] / (out[3] * sources) measures lane utilisation. */
@@ -480,6 +487,9 @@ int nf_stats_read(void *ws, int64_t *out, void *stream);
  *   out[2] = stages computed on the fast path (f = r^-3) and computed again on
  *            the exact path because a pair closer than eps_s met there
  *            (Eq. (spline)).
+ * out[0] and out[1] are those of the directed kernel's work list for this
+ * tuning, whichever kernel runs the box; out[2] counts what ran (the symmetric
+ * kernel's stage is a tile of 32 sources).
  * Returns NF_ERR_ARG for NULL pointers, NF_ERR_CUDA if a CUDA call fails. */
 int nf_stage_stats_read(void *ws, int64_t *out, void *stream);
 

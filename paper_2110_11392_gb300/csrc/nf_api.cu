@@ -138,6 +138,35 @@ int cuda_fail(cudaError_t e, const char* where)
 constexpr size_t kAlign = 256;
 size_t align_up(size_t x) { return (x + kAlign - 1) & ~(kAlign - 1); }
 
+// Which boxes the symmetric pair kernel runs (nf_sym.cu): those of the built-in
+// tuning of the direction with N within these.  From 64^3 particles on it is the
+// faster one (pair kernel, clustered: forward 0.89 against 0.99 ms, adjoint 1.59
+// against 1.80); a smaller box has too few pencils for its warps.  No box that
+// nf_forces_noalloc accepts is larger than 240k particles, so that entry point's
+// fixed scratch never has to hold the partial planes.  Above, the planes (18 slots
+// of 16 bytes a particle at R = 2) would take over 80 GB.  The time steps stay on
+// the directed kernel: the step size they write is a double made of a few of the
+// FP32 accelerations, read back by the next step, so the last bits of the sums
+// decide a run's trajectory, and a run continued with this version keeps it.
+constexpr int64_t kSymMinN = int64_t(1) << 18, kSymMaxN = int64_t(1) << 28;
+bool sym_box(int64_t N) { return N >= kSymMinN && N <= kSymMaxN; }
+// Tile groups of a dear pencil: the fewer pencils a warp has, the finer they are
+// cut (clustered 10^6 forward: 8 groups 3.59 ms, 4 3.88, 2 4.07; 200^3: 33.6, 33.4,
+// 33.1, where the combine's 0.94, 0.66, 0.52 ms for the slots weigh more).
+int sym_box_groups(int64_t N)
+{
+    return N < 1500000 ? 8 : N < (int64_t(1) << 22) ? 4 : N < (int64_t(1) << 25) ? 2 : 1;
+}
+bool same_tuning(const ForceTuning& a, const ForceTuning& b)
+{
+    return a.sinks_per_lane == b.sinks_per_lane && a.stage == b.stage && a.warps_per_block == b.warps_per_block &&
+           a.blocks_per_sm == b.blocks_per_sm;
+}
+bool sym_tuning(const ForceTuning& t, bool adjoint)
+{
+    return same_tuning(t, adjoint ? kBuiltinTuningAdj : kBuiltinTuning);
+}
+
 constexpr double kEpsRatio = 2.16;  // eps_s / eps_p, Sec. "Force Softening"
 
 struct Plan {
@@ -148,11 +177,13 @@ struct Plan {
     int max_R = 1;
     int max_nseg = 9;
     int nchunks = 0;     // combine chunks
+    bool any_sym = false;  // boxes that may run in the symmetric pair kernel
     SortPlan sp{};
     std::vector<BoxDev> boxes;
     // region offsets (bytes from ws)
     size_t o_boxes, o_keys_a, o_keys_b, o_rel_scratch, o_sort, o_off, o_rel, o_perm,
-        o_chunks, o_bucket_of, o_bucket_count, o_items, o_gs, o_partial, o_chunk_sums, o_step, total;
+        o_chunks, o_bucket_of, o_bucket_count, o_items, o_gs, o_partial, o_chunk_sums, o_step, o_sym, o_sym_dims,
+        o_sym_units, total;
     std::vector<size_t> guards;  // debug mode: guard block after each region
 };
 
@@ -213,12 +244,14 @@ int make_box(const nf_box& in, bool need_force, BoxDev* out)
     return NF_OK;
 }
 
-int make_plan(const nf_box* boxes, int nboxes, bool need_force, int chunk_lanes, Plan* p)
+// sym: boxes within the symmetric kernel's sizes run there (else all are directed)
+int make_plan(const nf_box* boxes, int nboxes, bool need_force, int chunk_lanes, Plan* p, bool sym = false)
 {
     if (!boxes || nboxes < 1) return fail(NF_ERR_ARG, "need at least one box");
     p->nboxes = nboxes;
     p->boxes.resize(nboxes);
-    int64_t N = 0, C = 0, items = 0, nchunks = 0;
+    int64_t N = 0, C = 0, items = 0, nchunks = 0, units = 0, planes = 0;
+    p->any_sym = false;
     int max_R = 1;
     for (int b = 0; b < nboxes; ++b) {
         int rc = make_box(boxes[b], need_force, &p->boxes[b]);
@@ -238,19 +271,37 @@ int make_plan(const nf_box* boxes, int nboxes, bool need_force, int chunk_lanes,
         C += cells;
         nchunks += (boxes[b].N + kCombineChunk - 1) / kCombineChunk;
         if (need_force) {
-            items += (2 * (int64_t)d.R + 1) * boxes[b].N / chunk_lanes + cells + 1;
             if (d.R > max_R) max_R = d.R;
+            if (sym && sym_box(d.N)) {
+                d.sym = 1;
+                d.groups = sym_box_groups(d.N);
+                units += sym_max_units(d.N, cells, d.R, d.groups);
+                p->any_sym = true;
+            }
+            items += (2 * (int64_t)d.R + 1) * boxes[b].N / chunk_lanes + cells + 1;
         }
         if (N >= (int64_t(1) << 31)) return fail(NF_ERR_ARG, "total N must be < 2^31");
         if (C >= (int64_t(1) << 31) - 1) return fail(NF_ERR_ARG, "total cells must be < 2^31");
     }
-    if (items >= (int64_t(1) << 31)) return fail(NF_ERR_ARG, "too many work items");
+    if (items >= (int64_t(1) << 31) || units >= (int64_t(1) << 31)) return fail(NF_ERR_ARG, "too many work items");
     p->N = N;
     p->C = C;
     p->max_items = items;
     p->max_R = max_R;
     p->max_nseg = (2 * max_R + 1) * (2 * max_R + 1);
     p->nchunks = (int)nchunks;
+    if (need_force) {
+        // partial sums: every particle's row (directed), then the planes of the symmetric boxes;
+        // a single box uses one or the other, so both start at the same place
+        const int64_t rows = 4 * (2 * (int64_t)max_R + 1) * N;
+        planes = rows;
+        for (BoxDev& d : p->boxes) {
+            if (!d.sym) continue;
+            const int64_t size = 4 * (int64_t)sym_slots(d.R, d.groups) * d.N;
+            d.plane_base = nboxes == 1 ? 0 : planes;
+            planes = std::max<int64_t>(planes, d.plane_base + size);
+        }
+    }
     p->sp = sort_plan(N, C);
 
     size_t o = 0;
@@ -280,11 +331,14 @@ int make_plan(const nf_box* boxes, int nboxes, bool need_force, int chunk_lanes,
         p->o_bucket_count = take(4 * kBuckets);
         p->o_items = take(16 * (size_t)items);
         p->o_gs = take(16 * (size_t)N);
-        p->o_partial = take(4 * 4 * (size_t)(2 * max_R + 1) * (size_t)N);
+        p->o_partial = take(4 * (size_t)planes);
+        p->o_sym = take(p->any_sym ? sizeof(SymCtl) + 16 * (size_t)nboxes : 16);
+        p->o_sym_dims = take(p->any_sym ? 8 * (size_t)C : 16);
+        p->o_sym_units = take(16 * (size_t)units + 16);
         p->o_chunk_sums = take(8 * 3 * (size_t)nchunks);
     } else {
         p->o_chunks = p->o_bucket_of = p->o_bucket_count = p->o_items = p->o_gs = p->o_partial =
-            p->o_chunk_sums = 0;
+            p->o_chunk_sums = p->o_sym = p->o_sym_dims = p->o_sym_units = 0;
     }
     p->total = o;
     return NF_OK;
@@ -382,23 +436,40 @@ int run_forces(const Plan& p, bool adjoint, const ForceTuning& t, const float* p
     unsigned* bucket_count = at<unsigned>(ws, p.o_bucket_count);
     NF_CUDA(cudaMemsetAsync(bucket_count, 0, 4 * kBuckets, s), "clear buckets");
     const int CH = 32 * t.sinks_per_lane;
-    NF_CUDA(launch_pencils(boxes, p.nboxes, (int)p.C, off, CH, t.stage, at<int>(ws, p.o_chunks), bucket_count,
-                           at<unsigned char>(ws, p.o_bucket_of), hdr, s),
+    SymCtl* sym = p.any_sym ? at<SymCtl>(ws, p.o_sym) : nullptr;
+    unsigned long long* sym_total = p.any_sym ? reinterpret_cast<unsigned long long*>(sym + 1) : nullptr;
+    const int gm = sym_gmax(adjoint);
+    int2* dims = p.any_sym ? at<int2>(ws, p.o_sym_dims) : nullptr;
+    int4* units = at<int4>(ws, p.o_sym_units);
+    int* chunks = at<int>(ws, p.o_chunks);
+    unsigned char* bucket_of = at<unsigned char>(ws, p.o_bucket_of);
+    if (p.any_sym) NF_CUDA(cudaMemsetAsync(sym, 0, sizeof(SymCtl) + 16 * (size_t)p.nboxes, s), "clear units");
+    NF_CUDA(launch_pencils(boxes, p.nboxes, (int)p.C, off, CH, t.stage, chunks, bucket_count, bucket_of, dims,
+                           sym_total, gm, hdr, s),
             "pencils");
-    NF_CUDA(launch_items(boxes, p.nboxes, (int)p.C, at<int>(ws, p.o_chunks), at<unsigned char>(ws, p.o_bucket_of),
-                         bucket_count, at<int4>(ws, p.o_items), hdr, s),
+    if (p.any_sym)
+        NF_CUDA(launch_sym_units(adjoint, boxes, p.nboxes, (int)p.C, off, dims, sym, sym_total, units, chunks,
+                                 bucket_of, bucket_count, hdr, s),
+                "symmetric work units");
+    NF_CUDA(launch_bucket_scan(bucket_count, hdr, s), "work items");
+    NF_CUDA(launch_items(boxes, p.nboxes, (int)p.C, chunks, bucket_of, bucket_count, at<int4>(ws, p.o_items), hdr, s),
             "work items");
     float4* gs = at<float4>(ws, p.o_gs);
     if (adjoint) NF_CUDA(launch_gather_g(g, perm, (int)p.N, gs, s), "gather g");
     float4* partial = at<float4>(ws, p.o_partial);
     const int pstride = 2 * p.max_R + 1;  // partial row of a particle: one float4 per pencil slot
     NF_CUDA(prof_mark(2, s), "profile");
+    if (p.any_sym)
+        NF_CUDA(launch_sym_force(adjoint, rho != nullptr, boxes, off, rel, gs, units, sym, hdr,
+                                 reinterpret_cast<float*>(partial), s),
+                adjoint ? "symmetric adjoint kernel" : "symmetric force kernel");
+    // (with nothing on its list where every box is symmetric)
     NF_CUDA(launch_force(adjoint, rho != nullptr, t, boxes, off, rel, gs, at<int4>(ws, p.o_items), hdr, partial,
                          pstride, p.max_nseg, s),
             adjoint ? "adjoint kernel" : "force kernel");
     NF_CUDA(prof_mark(3, s), "profile");
     double* chunk_sums = net ? at<double>(ws, p.o_chunk_sums) : nullptr;
-    NF_CUDA(launch_combine(adjoint, boxes, p.nboxes, p.nchunks, partial, pstride, out, rho, chunk_sums, s),
+    NF_CUDA(launch_combine(adjoint, boxes, p.nboxes, p.nchunks, partial, pstride, perm, out, rho, chunk_sums, s),
             "combine");
     if (net) NF_CUDA(launch_net(boxes, p.nboxes, chunk_sums, net, s), "net force");
     NF_CUDA(prof_mark(4, s), "profile");
@@ -437,7 +508,7 @@ int forces_entry(const nf_box* boxes, int nboxes, bool adjoint, const float* pos
     int rc = check_tuning(tune, &t, adjoint);
     if (rc) return rc;
     Plan p;
-    rc = make_plan(boxes, nboxes, true, 32 * t.sinks_per_lane, &p);
+    rc = make_plan(boxes, nboxes, true, 32 * t.sinks_per_lane, &p, sym_tuning(t, adjoint));
     if (rc) return rc;
     if (!pos || !out || (adjoint && !g)) return fail(NF_ERR_ARG, "null pointer argument");
     if (rho) {
@@ -492,6 +563,21 @@ int noalloc_scratch(void** out)
 }  // namespace
 }  // namespace nf
 
+namespace nf {
+namespace {
+
+// Workspace of a force call under any tuning: the directed plan with the most
+// items, or the plan with the symmetric kernel's planes.
+size_t force_workspace_bytes(const nf_box* boxes, int nboxes)
+{
+    Plan a, b;
+    if (make_plan(boxes, nboxes, true, 32, &a) || make_plan(boxes, nboxes, true, 32, &b, true)) return 0;
+    return a.total > b.total ? a.total : b.total;
+}
+
+}  // namespace
+}  // namespace nf
+
 using namespace nf;
 
 extern "C" {
@@ -504,16 +590,12 @@ size_t nf_workspace_bytes(int64_t N, int K, int R)
 {
     // the size does not depend on box or eps: use box 1 and a valid softening
     nf_box b = one_box(N, 1.0, K, R, K > 0 ? 0.5 / (kEpsRatio * K) : 1.0);
-    Plan p;
-    if (make_plan(&b, 1, true, 32, &p)) return 0;
-    return p.total;
+    return force_workspace_bytes(&b, 1);
 }
 
 size_t nf_workspace_bytes_batched(const nf_box* boxes, int nboxes)
 {
-    Plan p;
-    if (make_plan(boxes, nboxes, true, 32, &p)) return 0;
-    return p.total;
+    return force_workspace_bytes(boxes, nboxes);
 }
 
 int nf_bin(const float* pos, int64_t N, double box, int K, int32_t* cell_offsets, float* rel, int32_t* perm,
@@ -677,7 +759,7 @@ int nf_kdk_step(float* pos, float* vel, float* acc, int64_t N, double box, int K
     int rc = check_tuning(nullptr, &t);
     if (rc) return rc;
     Plan p;
-    rc = make_plan(&b, 1, true, 32 * t.sinks_per_lane, &p);
+    rc = make_plan(&b, 1, true, 32 * t.sinks_per_lane, &p);  // directed (see kSymMinN)
     if (rc) return rc;
     if (!pos || !vel || !acc || !dt) return fail(NF_ERR_ARG, "null pointer argument");
     if (prm && (!(prm->eta_acc > 0.0) || !(prm->hubble >= 0.0) || (prm->hubble > 0.0 && !(prm->eta_h > 0.0))))
@@ -1166,7 +1248,7 @@ int nf_forces_total(const float* pos, int64_t N, double box, int K, int R, doubl
     int rc = check_tuning(nullptr, &t);
     if (rc) return rc;
     Plan pn;
-    rc = make_plan(&b, 1, true, 32 * t.sinks_per_lane, &pn);
+    rc = make_plan(&b, 1, true, 32 * t.sinks_per_lane, &pn, sym_tuning(t, false));
     if (rc) return rc;
     if (!pos || !acc) return fail(NF_ERR_ARG, "null pointer argument");
     rc = check_ws(pn, ws, ws_bytes);
@@ -1195,7 +1277,7 @@ int nf_kdk_step_far(float* pos, float* vel, float* acc, int64_t N, double box, i
     int rc = check_tuning(nullptr, &t);
     if (rc) return rc;
     Plan pn;
-    rc = make_plan(&b, 1, true, 32 * t.sinks_per_lane, &pn);
+    rc = make_plan(&b, 1, true, 32 * t.sinks_per_lane, &pn);  // directed (see kSymMinN)
     if (rc) return rc;
     if (!pos || !vel || !acc || !dt) return fail(NF_ERR_ARG, "null pointer argument");
     if (prm && (!(prm->eta_acc > 0.0) || !(prm->hubble >= 0.0) || (prm->hubble > 0.0 && !(prm->eta_h > 0.0))))
@@ -1346,7 +1428,7 @@ int nf_stats_read(void* ws, int64_t* out, void* stream)
     e = cudaMemcpy(&h, ws, sizeof h, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(e, "stats read");
     out[0] = (int64_t)h.pairs;
-    out[1] = h.n_items;
+    out[1] = (int64_t)h.n_items + h.sym_units;
     out[2] = h.max_occ;
     out[3] = (int64_t)h.lane_pairs;
     return NF_OK;

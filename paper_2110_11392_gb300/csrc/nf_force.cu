@@ -48,42 +48,11 @@
 // on the tracked fast path like the rest of the first ring.
 #include <cuda_runtime.h>
 
-#include "nf_internal.cuh"
+#include "nf_pair.cuh"
 
 namespace nf {
 
 namespace {
-
-constexpr unsigned kFull = 0xffffffffu;
-constexpr float kTiny = 1e-25f;     // r^2 floor: coincident pairs stay finite (r^-3 < FLT_MAX)
-constexpr float kFarSrc = 1e18f;    // padding source coordinate: adds exactly 0
-constexpr float kFarSink = -1e18f;  // padding sink coordinate
-constexpr float kBig = 3.0e38f;
-
-__device__ __forceinline__ float rsqrt_approx(float x)
-{
-    float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-__device__ __forceinline__ int wrap(int a, int K)
-{
-    a %= K;
-    return a < 0 ? a + K : a;
-}
-
-__device__ __forceinline__ int find_box_by_cell(const BoxDev* boxes, int nboxes, int g)
-{
-    int lo = 0, hi = nboxes - 1;
-    while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        if (boxes[mid].cell_base <= g) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
-
 
 // Source cells of an item, (b, d) offsets in the plane, in rings around the
 // centre: the centre, its 8 neighbours, then rings 2, 3, 4 (the first
@@ -100,21 +69,6 @@ __constant__ signed char c_ring[81][2] = {
     {4, -4}, {4, -3}, {4, -2}, {4, -1}, {4, 0}, {4, 1}, {4, 2}, {4, 3}, {4, 4}};
 static_assert(NF_MAX_R <= 4, "the ring table covers R <= 4");
 
-__device__ __forceinline__ int cell_count(const int* off, int cid, int* start)
-{
-    int s = off[cid];
-    *start = s;
-    return off[cid + 1] - s;
-}
-
-__device__ __forceinline__ int cost_bucket(unsigned long long cost)
-{
-    if (cost == 0) return kBuckets - 1;
-    int h = (int)floorf(2.0f * log2f((float)cost));
-    int b = (kBuckets - 2) - h;
-    return b < 0 ? 0 : (b > kBuckets - 2 ? kBuckets - 2 : b);
-}
-
 // ---------------------------------------------------------------------------
 // Work list
 // ---------------------------------------------------------------------------
@@ -122,6 +76,7 @@ __device__ __forceinline__ int cost_bucket(unsigned long long cost)
 __global__ void k_pencils(const BoxDev* __restrict__ boxes, int nboxes, int Ctot,
                           const int* __restrict__ off, int CH, int SB, int* __restrict__ chunks,
                           unsigned* __restrict__ bucket_count, unsigned char* __restrict__ bucket_of,
+                          int2* __restrict__ sym_dims, unsigned long long* __restrict__ sym_total, int sym_gm,
                           WsHeader* hdr)
 {
     unsigned long long pairs = 0, lane_pairs = 0, stages = 0, stages_exact = 0;
@@ -130,7 +85,8 @@ __global__ void k_pencils(const BoxDev* __restrict__ boxes, int nboxes, int Ctot
     // 32), so the warp-wide votes below see all 32 lanes
     for (int gb = blockIdx.x * blockDim.x; gb < Ctot; gb += gridDim.x * blockDim.x) {
         const int g = gb + (int)threadIdx.x;
-        int nch = 0, bk = 0;
+        int nch = 0, bk = 0, box = -1;
+        unsigned long long scost = 0;
         if (g < Ctot) {
             const BoxDev& B = boxes[find_box_by_cell(boxes, nboxes, g)];
             const int K = B.K, R = B.R, cb = B.cell_base;
@@ -149,7 +105,6 @@ __global__ void k_pencils(const BoxDev* __restrict__ boxes, int nboxes, int Ctot
             int occ = cell_count(off, g, &st);
             max_occ = max(max_occ, occ);
             nch = (n_sink + CH - 1) / CH;
-            chunks[g] = nch;
             unsigned long long cost = (unsigned long long)n_src * (unsigned long long)min(n_sink, CH);
             bk = cost_bucket(cost);
             bucket_of[g] = (unsigned char)bk;
@@ -168,6 +123,31 @@ __global__ void k_pencils(const BoxDev* __restrict__ boxes, int nboxes, int Ctot
                 unsigned long long lanes = (unsigned long long)(nch - 1) * CH + 32ull * ((rem + 31) / 32);
                 lane_pairs += lanes * (unsigned long long)n_src;
             }
+            if (B.sym) {
+                // the symmetric kernel's pencil: the centre cell and half of the plane as sources
+                const int nb = 1 + ((2 * R + 1) * (2 * R + 1) - 1) / 2;
+                int n_half = 0;
+                for (int q = 0; q < nb; ++q)
+                    n_half += cell_count(off, cb + (i * K + wrap(j + c_half[q][0], K)) * K + wrap(k + c_half[q][1], K),
+                                         &st);
+                sym_dims[g] = make_int2(n_sink, n_half);
+                scost = sym_cost(n_sink, n_half, sym_gm);
+                box = find_box_by_cell(boxes, nboxes, g);
+                chunks[g] = nch;
+                nch = 0;  // on the directed list only if the box turns out directed (k_sym_count)
+            } else {
+                chunks[g] = nch;
+            }
+        }
+        // the symmetric boxes' total costs: one atomic per box per warp
+        if (sym_total) {
+            const unsigned same = __match_any_sync(kFull, box);
+            unsigned long long sum = 0;
+            for (int src = 0; src < 32; ++src) {
+                const unsigned long long v = __shfl_sync(kFull, scost, src);
+                if ((same >> src) & 1u) sum += v;
+            }
+            if (box >= 0 && (int)(threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(&sym_total[box], sum);
         }
         // one atomic per bucket per warp: most cells of a box fall in a few buckets
         const int key = nch ? bk : -1;
@@ -220,7 +200,8 @@ __global__ void k_items(const BoxDev* __restrict__ boxes, int nboxes, int Ctot,
     const int lane = threadIdx.x & 31;
     for (int gb = blockIdx.x * blockDim.x; gb < Ctot; gb += gridDim.x * blockDim.x) {
         const int g = gb + (int)threadIdx.x;
-        const int nch = g < Ctot ? chunks[g] : 0;
+        const int box = g < Ctot ? find_box_by_cell(boxes, nboxes, g) : 0;
+        const int nch = g < Ctot && !boxes[box].sym ? chunks[g] : 0;
         const int bk = nch ? (int)bucket_of[g] : -1;
         // one atomic per bucket per warp; each lane's chunks follow those of the
         // lanes below it in the same bucket (the order of items within a bucket
@@ -239,8 +220,7 @@ __global__ void k_items(const BoxDev* __restrict__ boxes, int nboxes, int Ctot,
         if (nch && lane == leader) base = atomicAdd(&cursor[bk], tot);
         base = __shfl_sync(kFull, base, leader) + pre;
         if (nch) {
-            const int b = find_box_by_cell(boxes, nboxes, g);
-            for (int q = 0; q < nch; ++q) items[base + q] = make_int4(g, q, b, 0);
+            for (int q = 0; q < nch; ++q) items[base + q] = make_int4(g, q, box, 0);
         }
     }
 }
@@ -257,19 +237,6 @@ __global__ void k_gather_g(const float* __restrict__ g, const int* __restrict__ 
 // ---------------------------------------------------------------------------
 // Pair arithmetic
 // ---------------------------------------------------------------------------
-
-struct Coef {
-    float c0, c1, c2;  // Eq. (spline) polynomial in cell units: c0 + r^2 (c2 + c1/r)
-    float e0, e1;      // f'(r)/r inside the softening: e1 + e0/r
-    float eps2;
-    int dens_defer;    // top hat only in stages where some lane met r < b
-};
-
-// Packed FP32x2 arithmetic (sm_100+ `add/mul/fma.rn.f32x2`): one instruction
-// works on the two halves of a 64-bit register pair.  The pair loops put two
-// sources side by side in each pair, so every instruction computes two
-// interactions of one sink; this halves the issue slots of the FP32 work.
-typedef unsigned long long f2;
 
 // Where r^-2 comes from in the fast paths: 1 = MUFU reciprocal, 0 = r^-1 * r^-1
 // on the FMA pipe.  Measured on GB300: the MUFU unit (16 lanes per clock per
@@ -304,70 +271,6 @@ constexpr int kAdjUnroll = NF_ADJ_UNROLL;
 constexpr int kFwdUnrollFar = NF_FWD_UNROLL_FAR;
 constexpr int kAdjUnrollFar = NF_ADJ_UNROLL_FAR;
 
-__device__ __forceinline__ f2 pk(float lo, float hi)
-{
-    f2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-// one half of a packed pair (the unpack names both halves; one is unused)
-#pragma nv_diag_suppress 550
-__device__ __forceinline__ float lo(f2 v)
-{
-    float a, b;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-    return a;
-}
-__device__ __forceinline__ float hi(f2 v)
-{
-    float a, b;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-    return b;
-}
-#pragma nv_diag_default 550
-__device__ __forceinline__ f2 add2(f2 a, f2 b)
-{
-    f2 d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2 mul2(f2 a, f2 b)
-{
-    f2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c)
-{
-    f2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ float rcp_approx(float x)
-{
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-__device__ __forceinline__ f2 rsqrt2(f2 v) { return pk(rsqrt_approx(lo(v)), rsqrt_approx(hi(v))); }
-// Smallest r^2 met so far, updated with both halves of a packed r^2: one
-// three-input min (sm_100 and later) instead of two.
-#ifndef NF_MIN3
-#define NF_MIN3 1
-#endif
-__device__ __forceinline__ float track_min(float t, f2 r2)
-{
-#if NF_MIN3
-    float m;
-    asm("min.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(t), "f"(lo(r2)), "f"(hi(r2)));
-    return m;
-#else
-    return fminf(t, fminf(lo(r2), hi(r2)));
-#endif
-}
-// r^-2 from the MUFU reciprocal: keeps the FMA pipe (the bottleneck) for the sums
-__device__ __forceinline__ f2 rcp2(f2 v) { return pk(rcp_approx(lo(v)), rcp_approx(hi(v))); }
-
 // Per-lane sink state.  Positions and gradients are held negated and
 // duplicated in both halves ({-x, -x}), so d = source + sink is one add2.
 template <int S>
@@ -390,13 +293,6 @@ struct StageView {
     const float4* GY;
     const float4* GZ;
 };
-
-// Top-hat density term of one packed pair (Sec. "Force Kernel"): b^2 - r^2 where positive.
-__device__ __forceinline__ f2 tophat2(f2 r2, f2 b2)
-{
-    const f2 t = fma2(r2, pk(-1.0f, -1.0f), b2);
-    return pk(fmaxf(lo(t), 0.0f), fmaxf(hi(t), 0.0f));
-}
 
 // Forward, fast path: f = r^-3 for every pair; TRK tracks the smallest r^2.
 // DENS adds the top-hat density estimate as a 4th sum.
@@ -613,15 +509,6 @@ struct WarpSmem {
         return raw_bytes + graw_bytes + soa_bytes + sh_bytes + ((t + 15) & ~size_t(15));
     }
 };
-
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc)
-{
-    unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
 struct ItemCtx {
     int K, R, cb;
@@ -972,14 +859,6 @@ k_force(const BoxDev* __restrict__ boxes, const int* __restrict__ off, const flo
 // constant, round once; the optional net force is an FP64 sum
 // ---------------------------------------------------------------------------
 
-// Error-free sum of two floats: s + e == a + b exactly (Knuth's TwoSum).
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e)
-{
-    s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-
 // One particle a thread: its row of partials is one round of independent
 // loads, so a small box (64^3: 1024 blocks) is as latency-hidden as a large
 // one.  Blocks of 4096 particles took 21 us for any box below 512k particles
@@ -987,11 +866,10 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e)
 // call of 4096 particles went from 171 to 158 us, of 32768 from 279 to 264.
 __global__ void __launch_bounds__(kCombineChunk)
 k_combine(const BoxDev* __restrict__ boxes, int nboxes, const float4* __restrict__ partial, int pstride,
-          float* __restrict__ out, float* __restrict__ rho, double* __restrict__ chunk_sums, bool adjoint)
+          const int* __restrict__ perm, float* __restrict__ out, float* __restrict__ rho,
+          double* __restrict__ chunk_sums, bool adjoint)
 {
-    // block = one chunk of particles (original order) of a single box; a
-    // particle's 2R+1 partials are one contiguous row, so the loads and the
-    // output rows of a warp are both contiguous
+    // block = one chunk of particles of a single box
     __shared__ double red[3][kCombineChunk / 32];
     int chunk = blockIdx.x;
     int lo = 0, hi = nboxes - 1;
@@ -1001,41 +879,83 @@ k_combine(const BoxDev* __restrict__ boxes, int nboxes, const float4* __restrict
         else hi = mid - 1;
     }
     const BoxDev& B = boxes[lo];
-    const int nslot = 2 * B.R + 1;
+    const int ns = 2 * B.R + 1;
     // the scale as an unevaluated float pair: scale = s_hi + s_lo to ~2^-48
     const float s_hi = adjoint ? B.grad_hi : B.acc_hi;
     const float s_lo = adjoint ? B.grad_lo : B.acc_lo;
     const bool out_aligned8 = (reinterpret_cast<uintptr_t>(out) & 7) == 0;
-    const int e = B.part_base + (chunk - B.chunk_base) * kCombineChunk + (int)threadIdx.x;
+    const int l = (chunk - B.chunk_base) * kCombineChunk + (int)threadIdx.x;
     double net[3] = {0.0, 0.0, 0.0};
-    constexpr int kMaxSlots = 2 * NF_MAX_R + 1;
-    if (e < B.part_base + B.N) {
-        const float4* row_in = partial + (size_t)e * (size_t)pstride;
-        // issue every partial load first (they are independent), then sum
-        float4 v[kMaxSlots];
+    if (l < B.N) {
+        // the partials, summed without rounding error into (sh, sl); .w the density
+        float sh[4] = {0.0f, 0.0f, 0.0f, 0.0f}, sl[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        auto add = [&](int c, float x) {
+            float t, err;
+            two_sum(sh[c], x, t, err);
+            sh[c] = t;
+            sl[c] = __fadd_rn(sl[c], err);
+        };
+        int e = B.part_base + l;
+        if (!B.sym) {
+            // original order: a particle's 2R+1 partials are one contiguous row, so the
+            // loads and the output rows of a warp are both contiguous
+            const float4* row_in = partial + (size_t)e * (size_t)pstride;
+            constexpr int kMaxSlots = 2 * NF_MAX_R + 1;
+            // issue every partial load first (they are independent), then sum
+            float4 v[kMaxSlots];
 #pragma unroll
-        for (int q = 0; q < kMaxSlots; ++q) v[q] = q < nslot ? row_in[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int q = 0; q < kMaxSlots; ++q) v[q] = q < ns ? row_in[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int q = 0; q < kMaxSlots; ++q) {
+                if (q < ns) {
+                    add(0, v[q].x);
+                    add(1, v[q].y);
+                    add(2, v[q].z);
+                    if (rho) add(3, v[q].w);
+                }
+            }
+        } else {
+            // sorted order: a slot's planes are contiguous across a warp
+            const int nslot = ns * B.groups + 1 + (ns * ns - 1) / 2;
+            const size_t N = (size_t)B.N;
+            const float* p = reinterpret_cast<const float*>(partial) + B.plane_base + l;
+            e = perm[B.part_base + l];
+            int q = 0;
+            constexpr int kU = 6;  // slots whose loads are in flight together
+            for (; q + kU <= nslot; q += kU) {
+                float v[kU][3];
+#pragma unroll
+                for (int u = 0; u < kU; ++u)
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) v[u][c] = p[(size_t)(3 * (q + u) + c) * N];
+#pragma unroll
+                for (int u = 0; u < kU; ++u)
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) add(c, v[u][c]);
+            }
+            for (; q < nslot; ++q)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) add(c, p[(size_t)(3 * q + c) * N]);
+            if (rho) {
+                const float* w = p + 3 * (size_t)nslot * N;
+                for (q = 0; q + kU <= nslot; q += kU) {
+                    float v[kU];
+#pragma unroll
+                    for (int u = 0; u < kU; ++u) v[u] = w[(size_t)(q + u) * N];
+#pragma unroll
+                    for (int u = 0; u < kU; ++u) add(3, v[u]);
+                }
+                for (; q < nslot; ++q) add(3, w[(size_t)q * N]);
+            }
+        }
         float a3[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            // the 2R+1 pencil partials, summed without rounding error into (sh, sl)
-            float sh = c == 0 ? v[0].x : (c == 1 ? v[0].y : v[0].z), sl = 0.0f;
-#pragma unroll
-            for (int q = 1; q < kMaxSlots; ++q) {
-                if (q < nslot) {
-                    const float x = c == 0 ? v[q].x : (c == 1 ? v[q].y : v[q].z);
-                    float t, err;
-                    two_sum(sh, x, t, err);
-                    sh = t;
-                    sl = __fadd_rn(sl, err);
-                }
-            }
             // (sh + sl) * (s_hi + s_lo), rounded once at the end
-            const float p = __fmul_rn(sh, s_hi);
-            const float perr = __fmaf_rn(sh, s_hi, -p);
-            const float a = __fadd_rn(p, __fmaf_rn(sh, s_lo, __fmaf_rn(sl, s_hi, perr)));
-            a3[c] = a;
-            if (chunk_sums) net[c] = B.mass * (double)a;
+            const float p = __fmul_rn(sh[c], s_hi);
+            const float perr = __fmaf_rn(sh[c], s_hi, -p);
+            a3[c] = __fadd_rn(p, __fmaf_rn(sh[c], s_lo, __fmaf_rn(sl[c], s_hi, perr)));
+            if (chunk_sums) net[c] = B.mass * (double)a3[c];
         }
         // the particle's row goes out in two stores (its 12 bytes start 8-byte
         // aligned for even e, 4 bytes past it for odd e)
@@ -1051,20 +971,8 @@ k_combine(const BoxDev* __restrict__ boxes, int nboxes, const float4* __restrict
             row[1] = a3[1];
             row[2] = a3[2];
         }
-        if (rho) {
-            // density partials (b^2 - r^2 sums), compensated, times 1/b^2
-            float sh = v[0].w, sl = 0.0f;
-#pragma unroll
-            for (int q = 1; q < kMaxSlots; ++q) {
-                if (q < nslot) {
-                    float t, err;
-                    two_sum(sh, v[q].w, t, err);
-                    sh = t;
-                    sl = __fadd_rn(sl, err);
-                }
-            }
-            rho[e] = __fmul_rn(__fadd_rn(sh, sl), B.dens_inv_b2);
-        }
+        // density partials (b^2 - r^2 sums), times 1/b^2
+        if (rho) rho[e] = __fmul_rn(__fadd_rn(sh[3], sl[3]), B.dens_inv_b2);
     }
     if (chunk_sums) {
         int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1193,14 +1101,17 @@ int force_blocks_per_sm(bool adjoint, bool density, const ForceTuning& t, int ma
 }
 
 cudaError_t launch_pencils(const BoxDev* boxes, int nboxes, int Ctot, const int* cell_off, int chunk, int stage,
-                           int* chunks, unsigned* bucket_count, unsigned char* bucket_of, WsHeader* hdr,
-                           cudaStream_t s)
+                           int* chunks, unsigned* bucket_count, unsigned char* bucket_of, int2* sym_dims,
+                           unsigned long long* sym_total, int sym_gm, WsHeader* hdr, cudaStream_t s)
 {
     k_pencils<<<grid_for(Ctot, 256), 256, 0, s>>>(boxes, nboxes, Ctot, cell_off, chunk, stage, chunks,
-                                                  bucket_count, bucket_of, hdr);
+                                                  bucket_count, bucket_of, sym_dims, sym_total, sym_gm, hdr);
     count_launches(1);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_bucket_scan(unsigned* bucket_count, WsHeader* hdr, cudaStream_t s)
+{
     k_bucket_scan<<<1, kBuckets, 0, s>>>(bucket_count, hdr);
     count_launches(1);
     return cudaGetLastError();
@@ -1248,10 +1159,10 @@ cudaError_t launch_force(bool adjoint, bool density, const ForceTuning& t, const
 }
 
 cudaError_t launch_combine(bool adjoint, const BoxDev* boxes, int nboxes, int nchunks, const float4* partial,
-                           int pstride, float* out, float* rho, double* chunk_sums, cudaStream_t s)
+                           int pstride, const int* perm, float* out, float* rho, double* chunk_sums, cudaStream_t s)
 {
     if (nchunks <= 0) return cudaSuccess;
-    k_combine<<<nchunks, kCombineChunk, 0, s>>>(boxes, nboxes, partial, pstride, out, rho, chunk_sums, adjoint);
+    k_combine<<<nchunks, kCombineChunk, 0, s>>>(boxes, nboxes, partial, pstride, perm, out, rho, chunk_sums, adjoint);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -10,7 +10,11 @@
 //   perm        int32 [N]       sorted slot -> particle (global index)
 //   items       int4 [<= M]     work items: (global centre cell, chunk, box, -)
 //   partial     float4 [N][2R+1]  per-pencil partial sums (ax, ay, az, density),
-//                                 one row per particle in original order
+//                                 one row per particle in original order; in a
+//                                 symmetric box (nf_sym.cu) instead float planes
+//                                 [slot][x, y, z][N] in sorted order, then the
+//                                 density's [slot][N]
+//   sym units   int4            work units of the symmetric boxes
 // A "global cell" numbers the cells of all boxes of a batch back to back:
 // box b owns cells [cell_base_b, cell_base_b + K_b^3).
 #pragma once
@@ -38,7 +42,6 @@ struct BoxDev {
     // as unevaluated float pairs (hi, lo), to 2^-48:
     float acc_hi, acc_lo;    // m / w^2: cell-unit pair sums -> box-unit acceleration
     float grad_hi, grad_lo;  // m / w^3: cell-unit Jacobian sums -> box-unit gradient
-    double pad;
     // Eq. (spline) in cell units: f(r) = min(c0 + r^2 (c2 + c1 / r), 1 / r^3)
     float c0, c1, c2;
     float eps2;      // eps_s^2 (cell units^2)
@@ -54,6 +57,13 @@ struct BoxDev {
     // 1: the top-hat term runs only in the pair-kernel stages where some pair
     // is closer than b (small b); 0: it is fused into every stage that can hold one
     int dens_defer;
+    // symmetric pair kernel (nf_sym.cu): 1 if it may run this box (cleared on the device where the
+    // directed one is the better, k_sym_choose); source-tile groups of a pencil
+    int sym;
+    int groups;
+    // first float of the box's planes of partial sums (symmetric)
+    long long plane_base;
+    double pad;
 };
 static_assert(sizeof(BoxDev) % 16 == 0, "BoxDev must stay 16-byte aligned");
 
@@ -67,7 +77,7 @@ struct WsHeader {
     unsigned long long lane_pairs;  // sink lanes issued * n_src
     // debug mode: byte offsets of the guard blocks that follow each workspace region
     int guard_count;
-    int pad0;
+    int sym_units;  // work units of the symmetric pair kernel
     long long guard_off[24];
     // pair-kernel stages: all, on the exact path from the start (the item's own
     // cell), and re-run on the exact path after the fast path met r < eps_s
@@ -87,6 +97,14 @@ struct BoxFill {
 
 constexpr int kCombineChunk = 256;   // particles per combine block, one a thread (never straddles boxes)
 constexpr int kBuckets = 64;         // cost buckets of the LPT work order
+
+// ---- symmetric pair kernel (nf_sym.cu) ----
+struct SymCtl {
+    unsigned bucket[kBuckets];
+    int queue;
+    int n_units;
+    int pad[62];
+};
 
 // Scratch of the time-step reduction (nf_step.cu).
 constexpr int kStepBlocks = 256;
@@ -236,9 +254,14 @@ struct ForceTuning {
     int blocks_per_sm;
 };
 
+// sym_dims, sym_total: of the boxes with .sym set, every pencil's (sinks, half-plane
+// sources) and the box's total cost (null when no box is symmetric); their chunks
+// are counted later, if the box turns out to be directed (launch_sym_units)
 cudaError_t launch_pencils(const BoxDev* boxes, int nboxes, int Ctot, const int* cell_off,
                            int chunk, int stage, int* chunks, unsigned* bucket_count,
-                           unsigned char* bucket_of, WsHeader* hdr, cudaStream_t s);
+                           unsigned char* bucket_of, int2* sym_dims, unsigned long long* sym_total,
+                           int sym_gmax, WsHeader* hdr, cudaStream_t s);
+cudaError_t launch_bucket_scan(unsigned* bucket_count, WsHeader* hdr, cudaStream_t s);
 cudaError_t launch_items(const BoxDev* boxes, int nboxes, int Ctot, const int* chunks,
                          const unsigned char* bucket_of, unsigned* bucket_count,
                          int4* items, WsHeader* hdr, cudaStream_t s);
@@ -248,13 +271,30 @@ cudaError_t launch_force(bool adjoint, bool density, const ForceTuning& t, const
                          const int* cell_off, const float4* rel, const float4* gs,
                          const int4* items, WsHeader* hdr, float4* partial, int pstride,
                          int max_nseg, cudaStream_t s);
-// partial rows of pstride float4 (2 max R + 1) per particle, original order
+// partial: rows of pstride float4 (2 max R + 1) per particle in original order (directed
+// boxes), or planes per slot and component in sorted order (symmetric ones)
 cudaError_t launch_combine(bool adjoint, const BoxDev* boxes, int nboxes, int nchunks,
-                           const float4* partial, int pstride, float* out,
+                           const float4* partial, int pstride, const int* perm, float* out,
                            float* rho, double* chunk_sums, cudaStream_t s);
 cudaError_t launch_net(const BoxDev* boxes, int nboxes, const double* chunk_sums,
                        double* net, cudaStream_t s);
 bool force_tuning_supported(const ForceTuning& t);
+
+// ---- symmetric pair kernel, work units, combine (nf_sym.cu) ----
+// partial slots of a particle: 2R+1 per group as a sink, the half plane's cells as a source
+int sym_slots(int R, int groups);
+int sym_gmax(bool adjoint);  // largest groups of a chunk
+long long sym_max_units(long long N, long long C, int R, int groups);
+// total: [2 nboxes], the boxes' costs and (written here) the costs of their dear pencils.
+// Clears .sym of the boxes that run better directed and adds their chunks to bucket_count.
+cudaError_t launch_sym_units(bool adjoint, BoxDev* boxes, int nboxes, int Ctot, const int* cell_off,
+                             const int2* dims, SymCtl* ctl, unsigned long long* total, int4* units,
+                             const int* chunks, const unsigned char* bucket_of, unsigned* bucket_count,
+                             WsHeader* hdr, cudaStream_t s);
+cudaError_t launch_sym_force(bool adjoint, bool density, const BoxDev* boxes, const int* cell_off, const float4* rel,
+                             const float4* gs, const int4* units, SymCtl* ctl, WsHeader* hdr, float* planes,
+                             cudaStream_t s);
+// planes: per box, slot q's x, y, z at plane_base + (3 q + c) N, its density at plane_base + (3 slots + q) N
 
 // ---- cell multipoles (nf_multipole.cu) ----
 int multipole_terms(int p);
