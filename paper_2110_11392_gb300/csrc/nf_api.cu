@@ -201,20 +201,15 @@ int make_box(const nf_box& in, bool need_force, BoxDev* out)
     b.N = (int)in.N;
     b.kl = (double)in.K / in.box;
     {
-        // short dyadic form of kl: then x * kl is exact in FP64 for any FP32 x
         int e = 0;
-        double f = std::frexp(b.kl, &e);                 // kl = f * 2^e, f in [0.5, 1)
-        long long m = (long long)std::ldexp(f, 53);      // exact 53-bit integer
-        int ex = e - 53;
-        while (m > 0 && (m & 1) == 0) {
-            m >>= 1;
-            ++ex;
+        const double f = std::frexp(b.kl, &e);  // kl = f * 2^e, f in [0.5, 1)
+        b.kl_mant = (unsigned long long)std::ldexp(f, 53);
+        b.kl_exp = e - 53;
+        if (b.kl > 1e-25 && b.kl < 1e25) {
+            b.kl_hi = (float)b.kl;
+            b.kl_lo = (float)(b.kl - (double)b.kl_hi);
         }
-        if (m > 0 && m < (1LL << 29)) {
-            b.kl_mant = (int)m;
-            b.kl_exp = ex;
-            if (m == 1 && ex >= -100 && ex <= 100) b.kl_pow2 = (float)b.kl;
-        }
+        if (f == 0.5 && e - 1 >= -100 && e - 1 <= 100) b.kl_pow2 = (float)b.kl;
     }
     const double w = in.box / in.K;
     const double scale_acc = 1.0 / ((double)in.N * w * w), scale_grad = 1.0 / ((double)in.N * w * w * w);
@@ -414,9 +409,11 @@ int run_binning(const Plan& p, const float* pos, void* ws, int32_t* cell_off, fl
         for (int q = 0; q < f.count; ++q) f.b[q] = p.boxes[first + q];
         NF_CUDA(launch_fill_boxes(f, boxes, s), "box table");
     }
+    bool pow2 = true;
+    for (const BoxDev& b : p.boxes) pow2 = pow2 && b.kl_pow2 != 0.0f;
     NF_CUDA(run_sort(p.sp, pos, (int)p.N, (int)p.C, boxes, p.nboxes, at<void>(ws, p.o_sort),
                      at<float4>(ws, p.o_rel_scratch), at<int>(ws, p.o_keys_a), at<int>(ws, p.o_keys_b), rel, perm,
-                     cell_off, hdr, s),
+                     cell_off, pow2, hdr, s),
             "binning sort");
     return NF_OK;
 }

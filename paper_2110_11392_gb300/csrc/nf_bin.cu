@@ -85,51 +85,73 @@ struct CellCoord {
     int bad;    // non-finite input
 };
 
-// The same function for any K / box and any x.  In integer arithmetic when
-// kl = kl_mant * 2^kl_exp with a short odd mantissa (the unit box: kl = K):
-// then t = x * kl, floor(t), t - c and (t - c) - 1/2 are all exact in FP64 for
-// 2^-29 <= |x| < 2^30, so the FP64 definition reduces to one rounding of an
-// exact value, which this path computes with 64-bit integers (the GPU's FP64
-// pipe is slow).  Other inputs take the FP64 path; both give identical
-// results.  Out of line: the sort passes inline only the power-of-two path of
-// cell_coord, which keeps their code (24 coordinates per thread) small.
-#ifndef NF_BIN_SLOW_NOINLINE
-#define NF_BIN_SLOW_NOINLINE 1
-#endif
-#if NF_BIN_SLOW_NOINLINE
-__device__ __noinline__
-#else
-__device__ __forceinline__
-#endif
-CellCoord cell_coord_general(float x, int K, int kl_mant, int kl_exp, double kl)
+// The same function for any K / box and any x, in integer arithmetic: the FP64
+// product t = RN53(x kl) of a 24-bit and a 53-bit mantissa is formed from two
+// 32-bit multiplies and rounded to nearest even; then floor(t), t - c and
+// (t - c) - 1/2 are integers over 2^s, and the offset is one rounding to 24 bits
+// (through 53 bits first where the FP64 difference is not exact, s >= 55).  GB300
+// runs FP64 at 1/64 of its FP32 rate, so the rule in doubles (cell_coord_fp64)
+// bounds the binning: 3 * 10^7 particles at K / box = 101 / 500 took 1333 us for the
+// cell ids and 1838 us for the first sort pass in doubles, 287 and 670 us this way
+// (and 96 and 461 us with the float pairs of cell_coord before it).
+// Takes 2^-10 <= t < 2^52 for x > 0 (2^-1 <= |t| for x < 0, below which 1 - |t| rounds);
+// the rest, zeros and subnormals go through doubles.  Both give the same bits.
+// Out of line: the sort passes inline only cell_coord's short paths, which keeps their code (24 coordinates per thread) small.
+template <bool OFF>
+__device__ __noinline__ CellCoord cell_coord_general(float x, int K, unsigned long long kl_mant, int kl_exp, double kl)
 {
+    typedef unsigned long long u64;
     CellCoord r;
     r.bad = 0;
+    r.off = 0.0f;
     const unsigned bits = __float_as_uint(x);
     const int E = (int)((bits >> 23) & 0xFF);
-    if (kl_mant > 0 && E >= 127 - 29 && E < 127 + 30) {
-        const long long P = (long long)((bits & 0x7FFFFFu) | 0x800000u) * (long long)kl_mant;
-        const int s = 150 - E - kl_exp;  // t = +-P * 2^-s
-        if (s >= 1 && s <= 53) {
-            const long long one = 1LL << s;
-            const long long low = P & (one - 1);
-            long long c;
-            long long frac;  // (t - c) * 2^s, in [0, 2^s)
-            if ((int)(bits >> 31) == 0) {
-                c = P >> s;
-                frac = low;
-            } else {
-                c = -(P >> s) - (low != 0);
+    const bool neg = (int)(bits >> 31) != 0;
+    if (E > 0 && E < 255) {
+        const unsigned mx = (bits & 0x7FFFFFu) | 0x800000u;
+        // P = mx * kl_mant = hi * 2^32 + lo, 2^75 <= P < 2^77
+        const u64 lo = (u64)mx * (unsigned)kl_mant;
+        const u64 hi = (u64)mx * (unsigned)(kl_mant >> 32) + (lo >> 32);
+        const int d = 23 + (int)(hi >> 44);  // bits beyond the 53rd
+        u64 q = (hi << (32 - d)) | ((unsigned)lo >> d);
+        const unsigned rem = (unsigned)lo << (32 - d);
+        q += rem > 0x80000000u || (rem == 0x80000000u && (q & 1u));
+        const int s = 150 - E - kl_exp - d;  // |t| = q * 2^-s
+        if (s >= 1 && s <= (neg ? 53 : 62)) {
+            const u64 one = 1ull << s;
+            const u64 low = q & (one - 1);
+            long long c = (long long)(q >> s);
+            u64 frac = low;  // (t - c) * 2^s
+            if (neg) {
+                c = -c - (low != 0);
                 frac = low ? one - low : 0;
             }
-            const long long o = frac - (one >> 1);
-            // exact scaling of the rounded integer by 2^-s
-            r.off = __ll2float_rn(o) * __int_as_float((127 - s) << 23);
+            if constexpr (OFF) {
+                const u64 half = one >> 1;
+                const bool below = frac < half;
+                u64 m = below ? half - frac : frac - half;  // |(t - c) - 1/2| * 2^s
+                if (s >= 55) {
+                    // m has s - 1 bits: the FP64 difference rounds to 53
+                    const int k = s - 54;
+                    const u64 rest = m & ((1ull << k) - 1), tie = 1ull << (k - 1);
+                    m >>= k;
+                    m += rest > tie || (rest == tie && (m & 1u));
+                    m <<= k;
+                }
+                if (m) {
+                    // to 24 bits from the leading 32, the bits below them in the last one
+                    const int lz = __clzll((long long)m);
+                    const u64 y = m << lz;
+                    const float f = __uint2float_rn((unsigned)(y >> 32) | (unsigned)((unsigned)y != 0u));
+                    const float v = f * __int_as_float((127 + 32 - lz - s) << 23);
+                    r.off = below ? -v : v;
+                }
+            }
             if (c >= 0 && c < K) {  // inside the box: no wrap (64-bit % is slow)
                 r.c = (int)c;
                 return r;
             }
-            long long cm = c % K;
+            const long long cm = c % K;
             r.c = (int)(cm < 0 ? cm + K : cm);
             return r;
         }
@@ -140,24 +162,55 @@ CellCoord cell_coord_general(float x, int K, int kl_mant, int kl_exp, double kl)
     return r;
 }
 
+// OFF off: the cell alone (*off is not written).  POW2: every box has K / box a
+// power of two.
+template <bool OFF, bool POW2>
 __device__ __forceinline__ int cell_coord(float x, const BoxDev& B, float* off, bool* bad)
 {
-    // K / box a power of two and x >= 0: t = x * K/box is exact in FP32 as in
+    // POW2 and x >= 0: t = x * K/box is exact in FP32 as in
     // FP64, so are c = floor(t) and t - c (for t >= 0), and one FP32
     // subtraction rounds (t - c) - 1/2 exactly as the FP64 rule's final
     // rounding does.  (For t < 0, t - floor(t) can round in FP32.)
-    if (B.kl_pow2 != 0.0f) {
+    if constexpr (POW2) {
         const float t = __fmul_rn(x, B.kl_pow2);
         if (t >= 0.0f && t < 1073741824.0f) {  // false for NaN
             const float c = floorf(t);
-            *off = __fsub_rn(__fsub_rn(t, c), 0.5f);
+            if constexpr (OFF) *off = __fsub_rn(__fsub_rn(t, c), 0.5f);
             const int ci = (int)c;
             if (ci < B.K) return ci;
             return ci % B.K;
         }
+    } else {
+        // Any other K / box: t = x K/box as a float pair p + e, within err of the FP64
+        // product (kl_hi + kl_lo is K / box to 2^-48).  p - c is exact and, unless p is an
+        // integer, inside (0, 1) by more than |e|, so c = floor(t).  The offset is the sum
+        // rounded to 24 bits, taken where no value within err rounds otherwise; the few
+        // others (near a rounding boundary, a face or a cell centre) take the integer path.
+        // A third of that path's instructions.
+        const float p = __fmul_rn(x, B.kl_hi);
+        if (p >= 0.000244140625f && p < 1048576.0f) {  // false for NaN and when kl_hi is 0
+            const float c = floorf(p), f = __fsub_rn(p, c);
+            const int ci = (int)c;
+            if constexpr (!OFF) {
+                if (f > 0.0f) return ci < B.K ? ci : ci % B.K;
+            } else {
+                const float e = __fmaf_rn(x, B.kl_lo, __fmaf_rn(x, B.kl_hi, -p));
+                const float a = __fsub_rn(f, 0.5f);
+                // f - 1/2 - a, exact: |f| <= 1/2 wherever a is rounded
+                const float tail = __fadd_rn(__fsub_rn(f, __fadd_rn(a, 0.5f)), e);
+                const float o = __fadd_rn(a, tail);
+                const float r = __fsub_rn(tail, __fsub_rn(o, a));
+                const float err = __fmaf_rn(p, 1.4210854715202004e-14f, 8.8817841970012523e-16f);  // 2^-46 p + 2^-50
+                if (f > 0.0f && fabsf(a) >= 0.000244140625f && __fadd_rn(o, __fadd_rn(r, err)) == o &&
+                    __fadd_rn(o, __fsub_rn(r, err)) == o) {
+                    *off = o;
+                    return ci < B.K ? ci : ci % B.K;
+                }
+            }
+        }
     }
-    const CellCoord r = cell_coord_general(x, B.K, B.kl_mant, B.kl_exp, B.kl);
-    *off = r.off;
+    const CellCoord r = cell_coord_general<OFF>(x, B.K, B.kl_mant, B.kl_exp, B.kl);
+    if constexpr (OFF) *off = r.off;
     if (r.bad) *bad = true;
     return r.c;
 }
@@ -170,16 +223,29 @@ __global__ void k_fill_boxes(BoxFill f, BoxDev* boxes)
 
 // Cell id (global: cell_base + local id) and cell-centred offsets of particle
 // e, whose coordinates are x[0..2].
+template <bool POW2>
 __device__ __forceinline__ int particle_key(const float* x, int e, const BoxDev* __restrict__ boxes, int nboxes,
                                            float4* rel, bool* bad)
 {
     const BoxDev& B = boxes[nboxes > 1 ? find_box(boxes, nboxes, e) : 0];
     float4 r;
-    const int cx = cell_coord(x[0], B, &r.x, bad);
-    const int cy = cell_coord(x[1], B, &r.y, bad);
-    const int cz = cell_coord(x[2], B, &r.z, bad);
+    const int cx = cell_coord<true, POW2>(x[0], B, &r.x, bad);
+    const int cy = cell_coord<true, POW2>(x[1], B, &r.y, bad);
+    const int cz = cell_coord<true, POW2>(x[2], B, &r.z, bad);
     r.w = __int_as_float(e);
     *rel = r;
+    return B.cell_base + (cx * B.K + cy) * B.K + cz;
+}
+
+// The cell id alone.
+template <bool POW2>
+__device__ __forceinline__ int particle_cell(const float* x, int e, const BoxDev* __restrict__ boxes, int nboxes,
+                                             bool* bad)
+{
+    const BoxDev& B = boxes[nboxes > 1 ? find_box(boxes, nboxes, e) : 0];
+    const int cx = cell_coord<false, POW2>(x[0], B, nullptr, bad);
+    const int cy = cell_coord<false, POW2>(x[1], B, nullptr, bad);
+    const int cz = cell_coord<false, POW2>(x[2], B, nullptr, bad);
     return B.cell_base + (cx * B.K + cy) * B.K + cz;
 }
 
@@ -239,7 +305,7 @@ __device__ __forceinline__ void stage_positions_warp(const float* __restrict__ p
 
 // Counts of every digit value in each tile, written to M[digit * tiles + tile].
 // FIRST computes the cell ids from the positions (and flags non-finite input).
-template <bool FIRST>
+template <bool FIRST, bool POW2>
 __global__ void __launch_bounds__(kSortWarps * 32)
 k_tile_hist(const float* __restrict__ pos, const BoxDev* __restrict__ boxes, int nboxes,
             const int* __restrict__ key_in, int N, int shift, int bits, int tiles, unsigned* __restrict__ M,
@@ -257,8 +323,7 @@ k_tile_hist(const float* __restrict__ pos, const BoxDev* __restrict__ boxes, int
     for (int l = threadIdx.x; l < n; l += blockDim.x) {
         int key;
         if constexpr (FIRST) {
-            float4 r;
-            key = particle_key(spos + 3 * l, (int)(base + l), boxes, nboxes, &r, &bad);
+            key = particle_cell<POW2>(spos + 3 * l, (int)(base + l), boxes, nboxes, &bad);
         } else {
             key = key_in[base + l];
         }
@@ -390,7 +455,7 @@ __host__ __device__ constexpr size_t sort_smem_bytes(int B)
 #ifndef NF_SORT_MINB
 #define NF_SORT_MINB 3
 #endif
-template <bool FIRST, bool LAST>
+template <bool FIRST, bool LAST, bool POW2>
 __global__ void __launch_bounds__(kSortWarps * 32, NF_SORT_MINB)
 k_sort_pass(const float* __restrict__ pos, const BoxDev* __restrict__ boxes, int nboxes,
             const float4* __restrict__ rel_in, const int* __restrict__ key_in, float4* __restrict__ rel_out,
@@ -437,7 +502,7 @@ k_sort_pass(const float* __restrict__ pos, const BoxDev* __restrict__ boxes, int
         if (l < n) {
             const int e = (int)(base + l);
             if constexpr (FIRST) {
-                key[r] = particle_key(spos + 3 * l, e, boxes, nboxes, &v[r], &bad);
+                key[r] = particle_key<POW2>(spos + 3 * l, e, boxes, nboxes, &v[r], &bad);
             } else {
                 v[r] = rel_in[e];
                 key[r] = key_in[e];
@@ -596,7 +661,7 @@ size_t sort_ctl_bytes(const SortPlan& p)
 
 cudaError_t run_sort(const SortPlan& p, const float* pos, int N, int C, const BoxDev* boxes, int nboxes,
                      void* ctl, float4* rel_scratch, int* key_a, int* key_b, float4* rel, int* perm, int* cell_off,
-                     WsHeader* hdr, cudaStream_t s)
+                     bool pow2, WsHeader* hdr, cudaStream_t s)
 {
     cudaError_t err;
     unsigned* M = static_cast<unsigned*>(ctl);
@@ -613,10 +678,10 @@ cudaError_t run_sort(const SortPlan& p, const float* pos, int N, int C, const Bo
         const int B = 1 << p.bits[k];
         const size_t mn = (size_t)p.tiles * B;
         if (first)
-            k_tile_hist<true><<<p.tiles, kSortWarps * 32, 0, s>>>(pos, boxes, nboxes, nullptr, N, p.shift[k],
-                                                                 p.bits[k], p.tiles, M, hdr);
+            (pow2 ? k_tile_hist<true, true> : k_tile_hist<true, false>)<<<p.tiles, kSortWarps * 32, 0, s>>>(
+                pos, boxes, nboxes, nullptr, N, p.shift[k], p.bits[k], p.tiles, M, hdr);
         else
-            k_tile_hist<false><<<p.tiles, kSortWarps * 32, 0, s>>>(pos, boxes, nboxes, kin, N, p.shift[k],
+            k_tile_hist<false, true><<<p.tiles, kSortWarps * 32, 0, s>>>(pos, boxes, nboxes, kin, N, p.shift[k],
                                                                   p.bits[k], p.tiles, M, hdr);
         count_launches(1);
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
@@ -629,8 +694,9 @@ cudaError_t run_sort(const SortPlan& p, const float* pos, int N, int C, const Bo
         const size_t smem = sort_smem_bytes(B);
         typedef void (*PassFn)(const float*, const BoxDev*, int, const float4*, const int*, float4*, int*, int*,
                                int, int, int, int, const unsigned*);
-        PassFn fn = first ? (last ? k_sort_pass<true, true> : k_sort_pass<true, false>)
-                          : (last ? k_sort_pass<false, true> : k_sort_pass<false, false>);
+        PassFn fn = !first  ? (last ? k_sort_pass<false, true, true> : k_sort_pass<false, false, true>)
+                    : pow2 ? (last ? k_sort_pass<true, true, true> : k_sort_pass<true, false, true>)
+                           : (last ? k_sort_pass<true, true, false> : k_sort_pass<true, false, false>);
         if ((err = ensure_smem((const void*)fn, (int)smem, true)) != cudaSuccess) return err;
         fn<<<p.tiles, kSortWarps * 32, smem, s>>>(pos, boxes, nboxes, rin, kin, rout, kout, perm, N, p.shift[k],
                                                   p.bits[k], p.tiles, M);

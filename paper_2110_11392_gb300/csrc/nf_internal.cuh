@@ -47,13 +47,16 @@ struct BoxDev {
     float eps2;      // eps_s^2 (cell units^2)
     // f'(r)/r inside the softening: e1 + e0 / r
     float e0, e1;
-    // K / box = kl_mant * 2^kl_exp with an odd kl_mant < 2^29, or kl_mant = 0
-    // when no such short form exists (then the shift stays in FP64)
-    int kl_mant, kl_exp;
+    // K / box = kl_mant * 2^kl_exp, 2^52 <= kl_mant < 2^53
+    unsigned long long kl_mant;
+    int kl_exp;
     // top-hat density estimate (Sec. "Force Kernel"): b^2 and 1/b^2 in cell units
     float dens_b2, dens_inv_b2;
     // K / box when it is a power of two (then x * K / box is exact in FP32), else 0
     float kl_pow2;
+    // K / box as a float pair, or 0 outside FP32's middle range
+    float kl_hi, kl_lo;
+    int pad[2];
     // 1: the top-hat term runs only in the pair-kernel stages where some pair
     // is closer than b (small b); 0: it is fused into every stage that can hold one
     int dens_defer;
@@ -63,7 +66,6 @@ struct BoxDev {
     int groups;
     // first float of the box's planes of partial sums (symmetric)
     long long plane_base;
-    double pad;
 };
 static_assert(sizeof(BoxDev) % 16 == 0, "BoxDev must stay 16-byte aligned");
 
@@ -244,7 +246,7 @@ size_t sort_ctl_bytes(const SortPlan& p);
 // and ctl (sort_ctl_bytes) are workspace; key_a ends with the sorted cell ids.
 cudaError_t run_sort(const SortPlan& p, const float* pos, int N, int C, const BoxDev* boxes, int nboxes,
                      void* ctl, float4* rel_scratch, int* key_a, int* key_b, float4* rel, int* perm, int* cell_off,
-                     WsHeader* hdr, cudaStream_t s);
+                     bool pow2, WsHeader* hdr, cudaStream_t s);  // pow2: every box's kl_pow2 is set
 
 // ---- work list, force, adjoint, combine (nf_force.cu) ----
 struct ForceTuning {
