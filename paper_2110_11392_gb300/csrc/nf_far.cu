@@ -57,7 +57,7 @@
 #include <tuple>
 #include <utility>
 
-#include "nf_internal.cuh"
+#include "nf_pair.cuh"
 
 namespace nf {
 
@@ -431,31 +431,6 @@ __device__ __forceinline__ dfl df_two_sum(float a, float b)
     return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
 }
 
-// a * z + t for a float z, without the final renormalisation: the result is
-// the unevaluated sum of TwoSum's high part and the collected error terms,
-// which a following step takes as it is (its exact product and TwoSum need
-// no normalised input).  Used inside Horner chains, where it saves three of
-// fourteen instructions per step.
-__device__ __forceinline__ dfl df_fma_f_nr(dfl a, float z, dfl t)
-{
-    const float p = __fmul_rn(a.h, z);
-    float e = __fmaf_rn(a.h, z, -p);
-    e = __fmaf_rn(a.l, z, e);
-    const dfl s = df_two_sum(p, t.h);
-    return {s.h, __fadd_rn(s.l, __fadd_rn(e, t.l))};
-}
-
-// a * b + t without the final renormalisation (see df_fma_f_nr)
-__device__ __forceinline__ dfl df_fma_nr(dfl a, dfl b, dfl t)
-{
-    const float p = __fmul_rn(a.h, b.h);
-    float e = __fmaf_rn(a.h, b.h, -p);
-    e = __fmaf_rn(a.h, b.l, e);
-    e = __fmaf_rn(a.l, b.h, e);
-    const dfl s = df_two_sum(p, t.h);
-    return {s.h, __fadd_rn(s.l, __fadd_rn(e, t.l))};
-}
-
 // a * b + t
 __device__ __forceinline__ dfl df_fma(dfl a, dfl b, dfl t)
 {
@@ -476,15 +451,6 @@ __device__ __forceinline__ dfl df_mul(dfl a, dfl b)
     return df_fast(p, e);
 }
 
-// a * z for a float z
-__device__ __forceinline__ dfl df_mul_f(dfl a, float z)
-{
-    const float p = __fmul_rn(a.h, z);
-    float e = __fmaf_rn(a.h, z, -p);
-    e = __fmaf_rn(a.l, z, e);
-    return df_fast(p, e);
-}
-
 __device__ __forceinline__ dfl df_add(dfl a, dfl b)
 {
     const dfl s = df_two_sum(a.h, b.h);
@@ -495,6 +461,57 @@ __device__ __forceinline__ dfl df_from(double v)
 {
     const float h = __double2float_rn(v);
     return {h, __double2float_rn(v - (double)h)};
+}
+
+// Two double-floats side by side (packed FP32x2 instructions), in half the issue
+// slots of two scalar ones.  ptxas fuses mul.rn.f32x2 with a following add.rn.f32x2 (it keeps
+// mul.rn.f32 apart), which would drop a product's rounding error; so a product is
+// an fma with the addend z0 = {-0, -0}, a value that only the launch knows.
+struct df2 {
+    f2 h, l;
+};
+__device__ __forceinline__ f2 neg2(f2 a) { return a ^ 0x8000000080000000ull; }
+__device__ __forceinline__ df2 df2_ld(float4 v) { return {pk(v.x, v.y), pk(v.z, v.w)}; }
+__device__ __forceinline__ float4 df2_st(df2 v) { return make_float4(lo(v.h), hi(v.h), lo(v.l), hi(v.l)); }
+// a * z + t for floats z (zn = -z), without the final renormalisation: the result is
+// the unevaluated sum of TwoSum's high part and the collected error terms,
+// which a following step takes as it is (its exact product and TwoSum need
+// no normalised input).  Used inside Horner chains, where it saves three of
+// fourteen instructions per step.
+__device__ __forceinline__ df2 df2_fma_f_nr(df2 a, f2 z, f2 zn, df2 t, f2 z0)
+{
+    const f2 p = fma2(a.h, z, z0);
+    const f2 q = fma2(a.l, zn, fma2(a.h, zn, p));  // minus the product's error terms
+    const f2 s = add2(p, t.h);
+    const f2 bb = sub2(s, p);
+    const f2 e = add2(sub2(p, sub2(s, bb)), sub2(t.h, bb));
+    return {s, add2(e, sub2(t.l, q))};
+}
+// a * b + t without the final renormalisation
+__device__ __forceinline__ df2 df2_fma_nr(df2 a, df2 b, df2 t, f2 z0)
+{
+    const f2 p = fma2(a.h, b.h, z0);
+    const f2 q = fma2(a.l, b.h, fma2(a.h, b.l, fma2(a.h, b.h, neg2(p))));
+    const f2 s = add2(p, t.h);
+    const f2 bb = sub2(s, p);
+    const f2 e = add2(sub2(p, sub2(s, bb)), sub2(t.h, bb));
+    return {s, add2(e, add2(q, t.l))};
+}
+// a * b
+__device__ __forceinline__ df2 df2_mul(df2 a, df2 b, f2 z0)
+{
+    const f2 p = fma2(a.h, b.h, z0);
+    const f2 q = fma2(a.l, b.h, fma2(a.h, b.l, fma2(a.h, b.h, neg2(p))));
+    const f2 s = add2(p, q);
+    return {s, sub2(q, sub2(s, p))};
+}
+// a * z for floats z
+__device__ __forceinline__ df2 df2_mul_f(df2 a, f2 z, f2 z0)
+{
+    const f2 p = fma2(a.h, z, z0);
+    const f2 q = fma2(a.l, z, fma2(a.h, z, neg2(p)));
+    const f2 s = add2(p, q);
+    return {s, sub2(q, sub2(s, p))};
 }
 
 // ---- double-float transforms and k-space product ---------------------------
@@ -776,18 +793,19 @@ __global__ void k_to_df(const double* __restrict__ src, long long n, dfl* __rest
 // Cell multipoles in cell units, double-float, folded onto the reduced basis
 // in the same kernel.  One block per cell and one thread per complete term:
 // kMpChunk particles at a time the block builds their powers x^e, y^e, z^e
-// (one thread per particle and axis) and the products x^a y^b (one per
-// particle and (a, b) pair) in shared memory, and each term thread adds
-// (x^a y^b) z^c to two double-float partial sums (updates without the
-// renormalisation, df_fma_nr; the partial sums are added with df_add, which
-// renormalises).  The cell's complete
+// (one thread per pair of particles and axis) and the products x^a y^b (one per
+// pair and (a, b)) in shared memory, and each term thread adds (x^a y^b) z^c of
+// a pair's two particles to two double-float partial sums, packed (updates
+// without the renormalisation, df2_fma_nr; the partial sums are added with
+// df_add, which renormalises).  Bound by its shared-memory reads (two 16-byte words
+// per pair and term, 86 % of the L1 throughput) and its barriers; unpacked it was
+// bound by instruction issue: 437 -> 365 us for 128^3 particles at order 8.  Two
+// terms of one (a, b) per thread (three words for two terms, half the threads)
+// measured 377 us, chunks of 64 and 128 particles 403 and 676 us.  The cell's complete
 // multipoles then go through the fold of k_far_reduce, Mr^r = sum_k
 // f_{r,k} M^k, with its coefficients as double-float pairs, and are written
 // as FP64 (Mr) or as double-float pairs (Mrd, for the double-float
-// transforms), with the cell's (0,0,2) term for its sum over cells.  (The
-// error-free transformations stay on scalar FP32 instructions: in probes the
-// packed .f32x2 form of the same sequence did not always keep the product's
-// rounding error, depending on the surrounding code.)
+// transforms), with the cell's (0,0,2) term for its sum over cells.
 #ifndef NF_MP_CHUNK
 #define NF_MP_CHUNK 32
 #endif
@@ -796,14 +814,16 @@ template <int P>
 __global__ void k_multipoles_red_df(const int* __restrict__ off, const float4* __restrict__ rel, int C,
                                     const int* __restrict__ rseg, const int* __restrict__ rk,
                                     const double* __restrict__ rcoef, double* __restrict__ Mr,
-                                    dfl* __restrict__ Mrd, double* __restrict__ m002)
+                                    dfl* __restrict__ Mrd, double* __restrict__ m002, float nz)
 {
     constexpr int P1 = P + 1, NAB = P1 * (P + 2) / 2, NT = far_terms(P), NR = P1 * P1;
-    extern __shared__ dfl smem_mp[];
+    constexpr int kPairs = kMpChunk / 2;
+    extern __shared__ __align__(16) float4 smem_mp[];
+    const f2 z0 = pk(nz, nz);
     const int nnz = rseg[NR];
-    dfl* pw = smem_mp;                                  // powers [3][kMpChunk][P1]
-    dfl* XY = pw + 3 * kMpChunk * P1;                   // products [kMpChunk][NAB]
-    dfl* Ms = XY + kMpChunk * NAB;                      // the cell's complete multipoles [NT]
+    float4* pw = smem_mp;                               // powers [3][kPairs][P1]: {h, h', l, l'} of a pair
+    float4* XY = pw + 3 * kPairs * P1;                  // products [kPairs][NAB]
+    dfl* Ms = reinterpret_cast<dfl*>(XY + kPairs * NAB);  // the cell's complete multipoles [NT]
     dfl* cf = Ms + NT;                                  // fold coefficients [nnz]
     int2* abt = reinterpret_cast<int2*>(cf + nnz);      // (a, b) of each product [NAB]
     int* ck = reinterpret_cast<int*>(abt + NAB);        // complete term of each coefficient [nnz]
@@ -825,46 +845,43 @@ __global__ void k_multipoles_red_df(const int* __restrict__ off, const float4* _
     const int t = threadIdx.x;
     if (t < NT) decode_term(t, P, a, b, c);
     const int ab = a * P1 - a * (a - 1) / 2 + b;
-    const dfl* Z = pw + 2 * kMpChunk * P1;
+    const float4* Z = pw + 2 * kPairs * P1;
     for (int cell = blockIdx.x; cell < C; cell += gridDim.x) {
         const int s0 = off[cell], s1 = off[cell + 1];
-        // two independent partial sums: a double-float update is a chain of
-        // dependent FP32 operations
-        dfl acc0 = {0.0f, 0.0f}, acc1 = {0.0f, 0.0f};
+        // two partial sums, of the even and the odd particles
+        df2 acc = {0ull, 0ull};
         for (int q0 = s0; q0 < s1; q0 += kMpChunk) {
-            const int nq = min(kMpChunk, s1 - q0);
+            const int nq = min(kMpChunk, s1 - q0), np = (nq + 1) >> 1;
             __syncthreads();  // the previous chunk (or the tables) are in place and read
-            for (int i = threadIdx.x; i < 3 * nq; i += blockDim.x) {
+            for (int i = threadIdx.x; i < 3 * np; i += blockDim.x) {
                 const int q = i / 3, d = i - 3 * q;
-                const float4 r4 = rel[q0 + q];
-                const float x = d == 0 ? r4.x : (d == 1 ? r4.y : r4.z);
-                dfl* row = pw + (d * kMpChunk + q) * P1;
-                dfl v = {x, 0.0f};
-                row[0] = dfl{1.0f, 0.0f};
-                if (P >= 1) row[1] = v;
+                const bool two = 2 * q + 1 < nq;
+                const float* r0 = reinterpret_cast<const float*>(rel + q0 + 2 * q);
+                const f2 x = pk(r0[d], two ? r0[4 + d] : 0.0f);
+                float4* row = pw + (d * kPairs + q) * P1;
+                // a missing second particle has x^0 = 0: all its products vanish
+                row[0] = make_float4(1.0f, two || d != 0 ? 1.0f : 0.0f, 0.0f, 0.0f);
+                df2 v = {x, 0ull};
+                if (P >= 1) row[1] = df2_st(v);
 #pragma unroll
                 for (int e = 2; e <= P; ++e) {
-                    v = df_mul_f(v, x);
-                    row[e] = v;
+                    v = df2_mul_f(v, x, z0);
+                    row[e] = df2_st(v);
                 }
             }
             __syncthreads();
-            for (int i = threadIdx.x; i < nq * NAB; i += blockDim.x) {
+            for (int i = threadIdx.x; i < np * NAB; i += blockDim.x) {
                 const int q = i / NAB, k = i - q * NAB;
                 const int2 ab2 = abt[k];
-                XY[q * NAB + k] = df_mul(pw[q * P1 + ab2.x], pw[(kMpChunk + q) * P1 + ab2.y]);
+                XY[q * NAB + k] =
+                    df2_st(df2_mul(df2_ld(pw[q * P1 + ab2.x]), df2_ld(pw[(kPairs + q) * P1 + ab2.y]), z0));
             }
             __syncthreads();
-            if (t < NT) {
-                int q = 0;
-                for (; q + 2 <= nq; q += 2) {
-                    acc0 = df_fma_nr(XY[q * NAB + ab], Z[q * P1 + c], acc0);
-                    acc1 = df_fma_nr(XY[(q + 1) * NAB + ab], Z[(q + 1) * P1 + c], acc1);
-                }
-                if (q < nq) acc0 = df_fma_nr(XY[q * NAB + ab], Z[q * P1 + c], acc0);
-            }
+            if (t < NT)
+                for (int q = 0; q < np; ++q)
+                    acc = df2_fma_nr(df2_ld(XY[q * NAB + ab]), df2_ld(Z[q * P1 + c]), acc, z0);
         }
-        if (t < NT) Ms[t] = df_add(acc0, acc1);
+        if (t < NT) Ms[t] = df_add(dfl{lo(acc.h), lo(acc.l)}, dfl{hi(acc.h), hi(acc.l)});
         __syncthreads();
         for (int r = threadIdx.x; r < NR; r += blockDim.x) {
             dfl m = {0.0f, 0.0f};
@@ -881,11 +898,15 @@ __global__ void k_multipoles_red_df(const int* __restrict__ off, const float4* _
 
 // The Taylor evaluation of k_taylor_forces in double-float: cell units, the
 // particle's stored FP32 offsets as the float multipliers of the Horner steps.
-// Each thread evaluates two particles at once (binned slots i and i + half):
-// a double-float Horner step is a chain of dependent FP32 operations, and two
-// independent chains keep the FP32 pipe busy.  The steps skip the
-// renormalisation (df_fma_f_nr, 11 instructions); the sums are converted to
-// FP64 as hi + lo at the end.
+// Each thread evaluates two particles at once (binned slots i and i + half) in the
+// halves of packed instructions: 11 per Horner step of both (df2_fma_f_nr, without
+// the renormalisation).  Scalar steps were bound by instruction issue (77 % of the
+// slots, with the coefficient loads) and by fetching their unrolled code: 462 us for
+// 128^3 particles at order 8.  Packed ones take 352 us, against 326 us that their
+// operations hold the FMA pipe (three of 2 x 3 operands, eight of 2 x 2 per step).
+// Blocks of 64 or 256 threads and more registers or fewer measured 355 to 390 us.  The coefficients
+// lie in two planes per cell, high parts and low parts, so that a load puts each
+// straight into its half.  The sums are converted to FP64 as hi + lo at the end.
 __device__ __forceinline__ void store_far(int orig, double ax, double ay, double az, double* __restrict__ acc_far,
                                           float* __restrict__ acc_add)
 {
@@ -901,75 +922,65 @@ __device__ __forceinline__ void store_far(int orig, double ax, double ay, double
     }
 }
 
-// The double-float Taylor evaluation's three Horner loops fully unrolled
-// (compile-time term offsets: no index arithmetic in the loop body), or not.
-#ifndef NF_TAYLOR_UNROLL
-#define NF_TAYLOR_UNROLL 1
-#endif
-#if NF_TAYLOR_UNROLL
-#define NF_TAYLOR_PRAGMA _Pragma("unroll")
-#else
-#define NF_TAYLOR_PRAGMA _Pragma("unroll 1")
-#endif
-
+constexpr int kTaylorThreads = 128;
 template <int P>
-__global__ void __launch_bounds__(128) k_taylor_forces_df(const int* __restrict__ cell, const float4* __restrict__ rel,
-                                                         const dfl* __restrict__ T, int N, int C, double scale,
-                                                         double* __restrict__ acc_far, float* __restrict__ acc_add)
+__global__ void __launch_bounds__(kTaylorThreads) k_taylor_forces_df(const int* __restrict__ cell, const float4* __restrict__ rel,
+                                                         const float* __restrict__ T, int N, double scale,
+                                                         double* __restrict__ acc_far, float* __restrict__ acc_add,
+                                                         float nz)
 {
     constexpr int NT = (P + 3) * (P + 2) * (P + 1) / 6;
-    const dfl zero = {0.0f, 0.0f};
+    const df2 zero = {0ull, 0ull};
+    const f2 z0 = pk(nz, nz);
     const int half = (N + 1) / 2;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < half; i += gridDim.x * blockDim.x) {
         const int j = i + half;                 // the second particle (may be past the end)
         const bool two = j < N;
         const int jj = two ? j : i;             // evaluate something valid, store only if two
         // the binning's sorted cell ids give each slot's cell (no search of the offsets)
-        const dfl* __restrict__ T0 = T + (size_t)cell[i] * NT;
-        const dfl* __restrict__ T1 = T + (size_t)cell[jj] * NT;
+        const float* __restrict__ T0 = T + (size_t)cell[i] * (2 * NT);
+        const float* __restrict__ T1 = T + (size_t)cell[jj] * (2 * NT);
         const float4 r0 = rel[i], r1 = rel[jj];
-        dfl F0 = zero, Fx0 = zero, Fy0 = zero, Fz0 = zero;
-        dfl F1 = zero, Fx1 = zero, Fy1 = zero, Fz1 = zero;
-NF_TAYLOR_PRAGMA
+        const f2 x = pk(r0.x, r1.x), y = pk(r0.y, r1.y), z = pk(r0.z, r1.z);
+        const f2 xn = neg2(x), yn = neg2(y), zn = neg2(z);
+        df2 F = zero, Fx = zero, Fy = zero, Fz = zero;
+        // the terms are taken from the last to the first, one after the other: for every a the
+        // rows b = P - a .. 0, which hold 1, 2, .. P - a + 1 terms in z.  The rows are unrolled
+        // and the loop over a is not: one straight body per row length (21 KB at P = 8).  All
+        // unrolled (88 KB) the warps waited for instructions half of their time.
+        const float* __restrict__ c0 = T0 + NT;
+        const float* __restrict__ c1 = T1 + NT;
+#pragma unroll 1
         for (int a = P; a >= 0; --a) {
-            const int base_a = NT - (P - a + 3) * (P - a + 2) * (P - a + 1) / 6;
-            dfl U0 = zero, Uy0 = zero, Uz0 = zero, U1 = zero, Uy1 = zero, Uz1 = zero;
-NF_TAYLOR_PRAGMA
-            for (int b = P - a; b >= 0; --b) {
-                const int base = base_a + b * (P - a + 1) - b * (b - 1) / 2;
-                dfl S0 = zero, Sz0 = zero, S1 = zero, Sz1 = zero;
-NF_TAYLOR_PRAGMA
-                for (int c = P - a - b; c >= 0; --c) {
-                    const float2 t0 = __ldg(reinterpret_cast<const float2*>(T0 + base + c));
-                    const float2 t1 = __ldg(reinterpret_cast<const float2*>(T1 + base + c));
-                    Sz0 = df_fma_f_nr(Sz0, r0.z, S0);
-                    Sz1 = df_fma_f_nr(Sz1, r1.z, S1);
-                    S0 = df_fma_f_nr(S0, r0.z, dfl{t0.x, t0.y});
-                    S1 = df_fma_f_nr(S1, r1.z, dfl{t1.x, t1.y});
+            df2 U = zero, Uy = zero, Uz = zero;
+#pragma unroll
+            for (int n = 1; n <= P + 1; ++n) {
+                c0 -= n;
+                c1 -= n;
+                df2 S = zero, Sz = zero;
+#pragma unroll
+                for (int c = n - 1; c >= 0; --c) {
+                    const df2 t = {pk(__ldg(c0 + c), __ldg(c1 + c)), pk(__ldg(c0 + NT + c), __ldg(c1 + NT + c))};
+                    Sz = df2_fma_f_nr(Sz, z, zn, S, z0);
+                    S = df2_fma_f_nr(S, z, zn, t, z0);
                 }
-                Uy0 = df_fma_f_nr(Uy0, r0.y, U0);
-                Uy1 = df_fma_f_nr(Uy1, r1.y, U1);
-                U0 = df_fma_f_nr(U0, r0.y, S0);
-                U1 = df_fma_f_nr(U1, r1.y, S1);
-                Uz0 = df_fma_f_nr(Uz0, r0.y, Sz0);
-                Uz1 = df_fma_f_nr(Uz1, r1.y, Sz1);
+                Uy = df2_fma_f_nr(Uy, y, yn, U, z0);
+                U = df2_fma_f_nr(U, y, yn, S, z0);
+                Uz = df2_fma_f_nr(Uz, y, yn, Sz, z0);
+                if (n == P - a + 1) break;
             }
-            Fx0 = df_fma_f_nr(Fx0, r0.x, F0);
-            Fx1 = df_fma_f_nr(Fx1, r1.x, F1);
-            F0 = df_fma_f_nr(F0, r0.x, U0);
-            F1 = df_fma_f_nr(F1, r1.x, U1);
-            Fy0 = df_fma_f_nr(Fy0, r0.x, Uy0);
-            Fy1 = df_fma_f_nr(Fy1, r1.x, Uy1);
-            Fz0 = df_fma_f_nr(Fz0, r0.x, Uz0);
-            Fz1 = df_fma_f_nr(Fz1, r1.x, Uz1);
+            Fx = df2_fma_f_nr(Fx, x, xn, F, z0);
+            F = df2_fma_f_nr(F, x, xn, U, z0);
+            Fy = df2_fma_f_nr(Fy, x, xn, Uy, z0);
+            Fz = df2_fma_f_nr(Fz, x, xn, Uz, z0);
         }
-        store_far(__float_as_int(r0.w), scale * ((double)Fx0.h + (double)Fx0.l),
-                  scale * ((double)Fy0.h + (double)Fy0.l), scale * ((double)Fz0.h + (double)Fz0.l), acc_far,
-                  acc_add);
+        store_far(__float_as_int(r0.w), scale * ((double)lo(Fx.h) + (double)lo(Fx.l)),
+                  scale * ((double)lo(Fy.h) + (double)lo(Fy.l)), scale * ((double)lo(Fz.h) + (double)lo(Fz.l)),
+                  acc_far, acc_add);
         if (two)
-            store_far(__float_as_int(r1.w), scale * ((double)Fx1.h + (double)Fx1.l),
-                      scale * ((double)Fy1.h + (double)Fy1.l), scale * ((double)Fz1.h + (double)Fz1.l), acc_far,
-                      acc_add);
+            store_far(__float_as_int(r1.w), scale * ((double)hi(Fx.h) + (double)hi(Fx.l)),
+                      scale * ((double)hi(Fy.h) + (double)hi(Fy.l)), scale * ((double)hi(Fz.h) + (double)hi(Fz.l)),
+                      acc_far, acc_add);
     }
 }
 
@@ -1042,7 +1053,7 @@ constexpr int kRebuildFetch = (kMaxFarOrder + 1) * (kMaxFarOrder + 1) / 32 + 1; 
 template <bool F64, bool DF, bool DIN>
 __global__ void k_far_rebuild(const void* __restrict__ Trv, int C, int p, int nt, int nr, const int4* __restrict__ ops,
                               const double2* __restrict__ opf, int t002, double lap, double t0_per_s002,
-                              const double* __restrict__ partial, double* __restrict__ T, dfl* __restrict__ Tdf)
+                              const double* __restrict__ partial, double* __restrict__ T, float* __restrict__ Tdf)
 {
     extern __shared__ int4 smem_rb[];
     int4* prog = smem_rb;                                     // [nt] ops
@@ -1136,7 +1147,11 @@ __global__ void k_far_rebuild(const void* __restrict__ Trv, int C, int p, int nt
         if (F64)
             for (int i = lane; i < nt; i += 32) T[(size_t)c * nt + i] = t[i];
         if (DF)
-            for (int i = lane; i < nt; i += 32) Tdf[(size_t)c * nt + i] = td[i];
+            for (int i = lane; i < nt; i += 32) {  // planes of high and low parts (k_taylor_forces_df)
+                float* o = Tdf + (size_t)c * (2 * nt) + i;
+                o[0] = td[i].h;
+                o[nt] = td[i].l;
+            }
         __syncwarp();  // the buffers are reused by the next cell
     }
 }
@@ -1705,7 +1720,7 @@ cudaError_t launch_multipoles_red_df(const int* off, const float4* rel, int C, i
         cudaError_t e = ensure_smem((const void*)k_multipoles_red_df<P>, (int)smem);                   \
         if (e != cudaSuccess) return e;                                                                \
         k_multipoles_red_df<P><<<grid, threads, smem, s>>>(off, rel, C, rseg, rk, rcoef, Mr,          \
-                                                           static_cast<dfl*>(Mrd), m002);              \
+                                                           static_cast<dfl*>(Mrd), m002, -0.0f);       \
         break;                                                                                         \
     }
         NF_MP_RED_CASE(0)
@@ -1732,13 +1747,13 @@ cudaError_t launch_multipoles_red_df(const int* off, const float4* rel, int C, i
 cudaError_t launch_taylor_forces_df(int p, const int* cell, const float4* rel, const void* Tdf, int N, int C,
                                     double scale, double* acc_far, float* acc_add, cudaStream_t s)
 {
-    const dfl* Td = static_cast<const dfl*>(Tdf);
-    const int need = ((N + 1) / 2 + 127) / 128;
+    const float* Td = static_cast<const float*>(Tdf);
+    const int need = ((N + 1) / 2 + kTaylorThreads - 1) / kTaylorThreads;
     const int grid = need < device_sms() * 16 ? need : device_sms() * 16;
     switch (p) {
 #define NF_TAYLOR_DF_CASE(P)                                                                        \
     case P:                                                                                         \
-        k_taylor_forces_df<P><<<grid, 128, 0, s>>>(cell, rel, Td, N, C, scale, acc_far, acc_add);   \
+        k_taylor_forces_df<P><<<grid, kTaylorThreads, 0, s>>>(cell, rel, Td, N, scale, acc_far, acc_add, -0.0f); \
         break;
         NF_TAYLOR_DF_CASE(0)
         NF_TAYLOR_DF_CASE(1)
@@ -1818,7 +1833,7 @@ cudaError_t launch_far_rebuild(const void* Tr, bool df_in, int C, int p, int nt,
     long long blocks = ((long long)C + kRebuildWarps - 1) / kRebuildWarps;  // one warp per cell
     const long long cap = (long long)device_sms() * (per_sm > 0 ? per_sm : 1);  // one wave, all resident
     if (blocks > cap) blocks = cap;
-    dfl* td = static_cast<dfl*>(Tdf);
+    float* td = static_cast<float*>(Tdf);
 #define NF_REBUILD_LAUNCH(A, B, D)                                                                           \
     k_far_rebuild<A, B, D><<<(int)blocks, kRebuildWarps * 32, smem, s>>>(Tr, C, p, nt, nr, ops, opf, t002, lap, \
                                                                         t0_per_s002, partial, T, td)

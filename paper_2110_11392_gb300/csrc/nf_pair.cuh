@@ -1,5 +1,5 @@
-// Device helpers shared by the pair kernels (nf_force.cu, nf_sym.cu): packed
-// FP32x2 arithmetic, asynchronous copies of the source stages, cell lookups.
+// Device helpers shared by the pair kernels (nf_force.cu, nf_sym.cu) and, for the
+// packed arithmetic, the far field (nf_far.cu): FP32x2 arithmetic, asynchronous copies of the source stages, cell lookups.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -113,6 +113,12 @@ __device__ __forceinline__ f2 add2(f2 a, f2 b)
 {
     f2 d;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 sub2(f2 a, f2 b)
+{
+    f2 d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
 __device__ __forceinline__ f2 mul2(f2 a, f2 b)
