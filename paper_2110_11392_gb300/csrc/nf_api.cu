@@ -138,18 +138,43 @@ int cuda_fail(cudaError_t e, const char* where)
 constexpr size_t kAlign = 256;
 size_t align_up(size_t x) { return (x + kAlign - 1) & ~(kAlign - 1); }
 
+// Work items of a box's directed list at most: every pencil's chunks.
+int64_t directed_items(int64_t N, int64_t C, int R, int chunk) { return (2 * (int64_t)R + 1) * N / chunk + C + 1; }
+
+// Net-force sums counted by nf_forces_noalloc's limit: one per 4096 particles.
+size_t limit_net_bytes(int64_t N) { return align_up(8 * 3 * (size_t)((N + 4095) / 4096)); }
+
+// Bytes of a box's directed plan in chunks of 128 sinks (make_plan's regions without
+// guards): what nf_forces_noalloc's fixed scratch is measured against.
+size_t directed_bytes(int64_t N, int64_t C, int R)
+{
+    static_assert(sizeof(BoxDev) <= 256, "one box takes one alignment unit");
+    const SortPlan sp = sort_plan(N, C);
+    size_t o = align_up(sizeof(WsHeader)) + align_up(sizeof(BoxDev));
+    for (size_t b : {4 * (size_t)N, 4 * (size_t)N, sp.passes > 1 ? 16 * (size_t)N : (size_t)16, sort_ctl_bytes(sp),
+                     4 * (size_t)(C + 1), 16 * (size_t)N, 4 * (size_t)N, sizeof(StepScratch), 4 * (size_t)C, (size_t)C,
+                     (size_t)4 * kBuckets, 16 * (size_t)directed_items(N, C, R, 128), 16 * (size_t)N,
+                     16 * (size_t)(2 * R + 1) * (size_t)N})
+        o += align_up(b);
+    return o + limit_net_bytes(N);
+}
+
 // Which boxes the symmetric pair kernel runs (nf_sym.cu): those of the built-in
-// tuning of the direction with N within these.  From 64^3 particles on it is the
-// faster one (pair kernel, clustered: forward 0.89 against 0.99 ms, adjoint 1.59
-// against 1.80); a smaller box has too few pencils for its warps.  No box that
-// nf_forces_noalloc accepts is larger than 240k particles, so that entry point's
-// fixed scratch never has to hold the partial planes.  Above, the planes (18 slots
-// of 16 bytes a particle at R = 2) would take over 80 GB.  The time steps stay on
-// the directed kernel: the step size they write is a double made of a few of the
-// FP32 accelerations, read back by the next step, so the last bits of the sums
-// decide a run's trajectory, and a run continued with this version keeps it.
+// tuning of the direction with N within these and too large for nf_forces_noalloc,
+// whose fixed scratch cannot hold the partial planes and whose results are
+// nf_forces'.  From 64^3 particles on it is the faster one (pair kernel, clustered:
+// forward 0.89 against 0.99 ms, adjoint 1.59 against 1.80); a smaller box has too few
+// pencils for its warps.  Above, the planes (18 slots of 16 bytes a particle at R = 2)
+// would take over 80 GB.  The time steps stay on the directed kernel: the step size
+// they write is a double made of a few of the FP32 accelerations, read back by the
+// next step, so the last bits of the sums decide a run's trajectory, and a run
+// continued with this version keeps it.
 constexpr int64_t kSymMinN = int64_t(1) << 18, kSymMaxN = int64_t(1) << 28;
-bool sym_box(int64_t N) { return N >= kSymMinN && N <= kSymMaxN; }
+bool sym_box(const nf_box& b)
+{
+    return b.N >= kSymMinN && b.N <= kSymMaxN &&
+           directed_bytes(b.N, (int64_t)b.K * b.K * b.K, b.R) > (size_t)NF_NOALLOC_SCRATCH_BYTES;
+}
 // Tile groups of a dear pencil: the fewer pencils a warp has, the finer they are
 // cut (clustered 10^6 forward: 8 groups 3.59 ms, 4 3.88, 2 4.07; 200^3: 33.6, 33.4,
 // 33.1, where the combine's 0.94, 0.66, 0.52 ms for the slots weigh more).
@@ -267,13 +292,13 @@ int make_plan(const nf_box* boxes, int nboxes, bool need_force, int chunk_lanes,
         nchunks += (boxes[b].N + kCombineChunk - 1) / kCombineChunk;
         if (need_force) {
             if (d.R > max_R) max_R = d.R;
-            if (sym && sym_box(d.N)) {
+            if (sym && sym_box(boxes[b])) {
                 d.sym = 1;
                 d.groups = sym_box_groups(d.N);
                 units += sym_max_units(d.N, cells, d.R, d.groups);
                 p->any_sym = true;
             }
-            items += (2 * (int64_t)d.R + 1) * boxes[b].N / chunk_lanes + cells + 1;
+            items += directed_items(d.N, cells, d.R, chunk_lanes);
         }
         if (N >= (int64_t(1) << 31)) return fail(NF_ERR_ARG, "total N must be < 2^31");
         if (C >= (int64_t(1) << 31) - 1) return fail(NF_ERR_ARG, "total cells must be < 2^31");
@@ -327,9 +352,9 @@ int make_plan(const nf_box* boxes, int nboxes, bool need_force, int chunk_lanes,
         p->o_items = take(16 * (size_t)items);
         p->o_gs = take(16 * (size_t)N);
         p->o_partial = take(4 * (size_t)planes);
-        p->o_sym = take(p->any_sym ? sizeof(SymCtl) + 16 * (size_t)nboxes : 16);
-        p->o_sym_dims = take(p->any_sym ? 8 * (size_t)C : 16);
-        p->o_sym_units = take(16 * (size_t)units + 16);
+        p->o_sym = p->any_sym ? take(sizeof(SymCtl) + 16 * (size_t)nboxes) : 0;
+        p->o_sym_dims = p->any_sym ? take(8 * (size_t)C) : 0;
+        p->o_sym_units = p->any_sym ? take(16 * (size_t)units) : 0;
         p->o_chunk_sums = take(8 * 3 * (size_t)nchunks);
     } else {
         p->o_chunks = p->o_bucket_of = p->o_bucket_count = p->o_items = p->o_gs = p->o_partial =
@@ -536,7 +561,10 @@ namespace {
 // stand-in); its device address comes from cudaGetSymbolAddress, looked up
 // once per device with that device current and then reused.
 constexpr int kMaxDevices = 64;
-static __device__ __align__(256) unsigned char g_noalloc_scratch[NF_NOALLOC_SCRATCH_BYTES];
+// (Its limit counts a net-force sum per 4096 particles; the sums per kCombineChunk take
+// less than kNoallocSlack beyond that at the limit.)
+constexpr size_t kNoallocSlack = size_t(1) << 18;
+static __device__ __align__(256) unsigned char g_noalloc_scratch[NF_NOALLOC_SCRATCH_BYTES + kNoallocSlack];
 std::mutex g_noalloc_mutex;
 void* g_noalloc_ptr[kMaxDevices] = {};
 
@@ -711,16 +739,17 @@ int nf_forces_noalloc(const float* pos, int64_t N, double box, int K, int R, dou
     rc = make_plan(&b, 1, true, 32 * t.sinks_per_lane, &p);
     if (rc) return rc;
     if (!pos || !acc) return fail(NF_ERR_ARG, "null pointer argument");
-    if (p.total > (size_t)NF_NOALLOC_SCRATCH_BYTES)
+    const size_t need = p.total - align_up(8 * 3 * (size_t)p.nchunks) + limit_net_bytes(N);
+    if (need > (size_t)NF_NOALLOC_SCRATCH_BYTES)
         return fail(NF_ERR_WORKSPACE,
                     "nf_forces_noalloc: N = %lld, K = %d, R = %d needs %zu bytes of scratch, more than the "
                     "library's fixed %u-byte array; call nf_forces with a workspace instead",
-                    (long long)N, K, R, p.total, (unsigned)NF_NOALLOC_SCRATCH_BYTES);
+                    (long long)N, K, R, need, (unsigned)NF_NOALLOC_SCRATCH_BYTES);
     void* scratch = nullptr;
     rc = noalloc_scratch(&scratch);
     if (rc) return rc;
-    return forces_entry(&b, 1, false, pos, nullptr, acc, net, nullptr, scratch, NF_NOALLOC_SCRATCH_BYTES,
-                        stream);
+    return forces_entry(&b, 1, false, pos, nullptr, acc, net, nullptr, scratch,
+                        (size_t)NF_NOALLOC_SCRATCH_BYTES + kNoallocSlack, stream);
 }
 
 int nf_timestep(const float* pos, const float* vel, const float* acc, int64_t N, double box, int K,
