@@ -182,12 +182,26 @@ int sym_box_groups(int64_t N)
 {
     return N < 1500000 ? 8 : N < (int64_t(1) << 22) ? 4 : N < (int64_t(1) << 25) ? 2 : 1;
 }
+// Warps that share an item of the directed kernel, by the items of the call's boxes
+// at mean occupancy.  With fewer items than warps on the chip a call takes as long
+// as its dearest item; sharing costs a barrier per round of stages and the idle
+// warps of the last round, and does not change a bit of the results.  Whole calls,
+// one warp against the choice: forward 4096 particles (250 items) 169 -> 92 us,
+// 16384 (648) 305 -> 158, 32768 uniform and clustered (1536) 263 -> 211 and 438 -> 219,
+// 65536 clustered (3000) 516 -> 374, 131072 clustered (6591) 717 -> 640, 230000 (10125)
+// 938 against 998 with four; adjoint 174 -> 111, 290 -> 234, 373 -> 342, and 602 against
+// 631 with four at 3000 items.
+int coop_warps(int64_t items, bool adjoint)
+{
+    if (adjoint) return items < 2000 ? 4 : 1;
+    return items < 1000 ? 8 : items < 8000 ? 4 : 1;
+}
 bool same_tuning(const ForceTuning& a, const ForceTuning& b)
 {
     return a.sinks_per_lane == b.sinks_per_lane && a.stage == b.stage && a.warps_per_block == b.warps_per_block &&
            a.blocks_per_sm == b.blocks_per_sm;
 }
-bool sym_tuning(const ForceTuning& t, bool adjoint)
+bool builtin_tuning(const ForceTuning& t, bool adjoint)
 {
     return same_tuning(t, adjoint ? kBuiltinTuningAdj : kBuiltinTuning);
 }
@@ -199,6 +213,7 @@ struct Plan {
     int64_t N = 0;       // total particles
     int64_t C = 0;       // total cells
     int64_t max_items = 0;
+    int64_t mean_items = 0;  // work items if every cell held its box's mean occupancy
     int max_R = 1;
     int max_nseg = 9;
     int nchunks = 0;     // combine chunks
@@ -272,6 +287,7 @@ int make_plan(const nf_box* boxes, int nboxes, bool need_force, int chunk_lanes,
     p->boxes.resize(nboxes);
     int64_t N = 0, C = 0, items = 0, nchunks = 0, units = 0, planes = 0;
     p->any_sym = false;
+    p->mean_items = 0;
     int max_R = 1;
     for (int b = 0; b < nboxes; ++b) {
         int rc = make_box(boxes[b], need_force, &p->boxes[b]);
@@ -299,6 +315,7 @@ int make_plan(const nf_box* boxes, int nboxes, bool need_force, int chunk_lanes,
                 p->any_sym = true;
             }
             items += directed_items(d.N, cells, d.R, chunk_lanes);
+            p->mean_items += cells * (((2 * (int64_t)d.R + 1) * d.N / cells + chunk_lanes - 1) / chunk_lanes);
         }
         if (N >= (int64_t(1) << 31)) return fail(NF_ERR_ARG, "total N must be < 2^31");
         if (C >= (int64_t(1) << 31) - 1) return fail(NF_ERR_ARG, "total cells must be < 2^31");
@@ -486,7 +503,8 @@ int run_forces(const Plan& p, bool adjoint, const ForceTuning& t, const float* p
                                  reinterpret_cast<float*>(partial), s),
                 adjoint ? "symmetric adjoint kernel" : "symmetric force kernel");
     // (with nothing on its list where every box is symmetric)
-    NF_CUDA(launch_force(adjoint, rho != nullptr, t, boxes, off, rel, gs, at<int4>(ws, p.o_items), hdr, partial,
+    const int coop = builtin_tuning(t, adjoint) && !p.any_sym ? coop_warps(p.mean_items, adjoint) : 1;
+    NF_CUDA(launch_force(adjoint, rho != nullptr, t, coop, boxes, off, rel, gs, at<int4>(ws, p.o_items), hdr, partial,
                          pstride, p.max_nseg, s),
             adjoint ? "adjoint kernel" : "force kernel");
     NF_CUDA(prof_mark(3, s), "profile");
@@ -530,7 +548,7 @@ int forces_entry(const nf_box* boxes, int nboxes, bool adjoint, const float* pos
     int rc = check_tuning(tune, &t, adjoint);
     if (rc) return rc;
     Plan p;
-    rc = make_plan(boxes, nboxes, true, 32 * t.sinks_per_lane, &p, sym_tuning(t, adjoint));
+    rc = make_plan(boxes, nboxes, true, 32 * t.sinks_per_lane, &p, builtin_tuning(t, adjoint));
     if (rc) return rc;
     if (!pos || !out || (adjoint && !g)) return fail(NF_ERR_ARG, "null pointer argument");
     if (rho) {
@@ -1274,7 +1292,7 @@ int nf_forces_total(const float* pos, int64_t N, double box, int K, int R, doubl
     int rc = check_tuning(nullptr, &t);
     if (rc) return rc;
     Plan pn;
-    rc = make_plan(&b, 1, true, 32 * t.sinks_per_lane, &pn, sym_tuning(t, false));
+    rc = make_plan(&b, 1, true, 32 * t.sinks_per_lane, &pn, builtin_tuning(t, false));
     if (rc) return rc;
     if (!pos || !acc) return fail(NF_ERR_ARG, "null pointer argument");
     rc = check_ws(pn, ws, ws_bytes);

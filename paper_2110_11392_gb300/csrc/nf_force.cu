@@ -548,9 +548,11 @@ struct WarpBufs {
     float4* graw;   // [2][B] (adjoint)
     float* soa;     // [NC][B]
     float2* sh;     // [2][B]
+    float* stage_sums;  // cooperative items: [W][sums][32], the warps' sums of one round of stages
+    float* totals;      // and [sums][32], the item's
 };
 
-template <int S, int B, bool ADJ, bool DENS>
+template <int S, int B, bool ADJ, bool DENS, int W = 1>
 __device__ __forceinline__ void run_item(const ItemCtx& it, const Coef& cf, f2 b2,
                                          const float4* __restrict__ rel, const float4* __restrict__ gs,
                                          const WarpBufs& wb, const int* seg_pre,
@@ -643,77 +645,119 @@ __device__ __forceinline__ void run_item(const ItemCtx& it, const Coef& cf, f2 b
         }
     };
 
-    if (nst > 0) issue(0, 0);
-    for (int st = 0; st < nst; ++st) {
-        const int buf = st & 1;
-        if (st + 1 < nst) {
-            issue(st + 1, buf ^ 1);
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
-        }
-        fixup(buf);
-        __syncwarp();
-        int beg, end;
-        stage_range(st, beg, end);
-        const int cnt = (end - beg + 7) & ~7;
-        const float* soa = wb.soa;
-        StageView v;
-        v.X = reinterpret_cast<const float4*>(soa + 0 * B);
-        v.Y = reinterpret_cast<const float4*>(soa + 1 * B);
-        v.Z = reinterpret_cast<const float4*>(soa + 2 * B);
-        v.GX = reinterpret_cast<const float4*>(soa + (ADJ ? 3 : 0) * B);
-        v.GY = reinterpret_cast<const float4*>(soa + (ADJ ? 4 : 0) * B);
-        v.GZ = reinterpret_cast<const float4*>(soa + (ADJ ? 5 : 0) * B);
-        // the centre cell's stages hold the self pairs only for chunks with sinks
-        // in that cell; other chunks run them on the tracked fast path
-        bool exact = it.has_self && st < nst0;
-        // Sources of ring 2 and beyond are at least one cell away from every
-        // sink of the pencil, and every source is more than one cell away from
-        // the sinks of cells two or more cells from the plane in x: the top hat
-        // (b <= one cell) and the softened branch (eps_s <= one cell) cannot
-        // occur there.
-        const bool far = beg >= it.n_near || !it.near_x;
-        const bool dens = DENS && (!dens_near_only || !far);
-        if (!exact) {
-#pragma unroll
-            for (int s = 0; s < S; ++s) k.sx[s] = k.sy[s] = k.sz[s] = k.sw[s] = 0ull;
-            float trk = kBig;
-            if (far && soft_near_only) {
-                if constexpr (ADJ) stage_adj_fast<S, false>(v, cnt, k, trk);
-                else if (dens) stage_fwd_fast<S, DENS, false>(v, cnt, k, trk, b2);
-                else stage_fwd_fast<S, false, false>(v, cnt, k, trk, b2);
+    // W > 1: the W warps of the block share the item and take its stages in turn; their stage
+    // sums are added to the totals in stage order, as one warp adds them, so the bits do not
+    // depend on W
+    constexpr int NS = DENS ? 4 : 3;
+    const int w = W > 1 ? (int)threadIdx.x >> 5 : 0;
+    if constexpr (W > 1)
+        for (int q = w; q < NS * S; q += W) wb.totals[q * 32 + lane] = 0.0f;
+    if (w < nst) issue(w, 0);
+    for (int st0 = 0; st0 < nst; st0 += W) {
+        const int st = st0 + w;
+        const int buf = (st0 / W) & 1;
+        if (W == 1 || st < nst) {
+            if (st + W < nst) {
+                issue(st + W, buf ^ 1);
+                cp_async_wait<1>();
             } else {
-                if constexpr (ADJ) stage_adj_fast<S>(v, cnt, k, trk);
-                else if (dens && !dens_defer) stage_fwd_fast<S, DENS>(v, cnt, k, trk, b2);
-                else stage_fwd_fast<S, false>(v, cnt, k, trk, b2);
-                exact = __any_sync(kFull, trk < cf.eps2);
-                if (exact && lane == 0) atomicAdd(&hdr->stages_rerun, 1ull);  // rare
-                if constexpr (DENS && !ADJ) {
-                    // a pair closer than b gives a positive term; elsewhere every term is +0
-                    if (dens && dens_defer && !exact && __any_sync(kFull, trk < lo(b2)))
-                        stage_density<S>(v, cnt, k, b2);
+                cp_async_wait<0>();
+            }
+            fixup(buf);
+            __syncwarp();
+            int beg, end;
+            stage_range(st, beg, end);
+            const int cnt = (end - beg + 7) & ~7;
+            const float* soa = wb.soa;
+            StageView v;
+            v.X = reinterpret_cast<const float4*>(soa + 0 * B);
+            v.Y = reinterpret_cast<const float4*>(soa + 1 * B);
+            v.Z = reinterpret_cast<const float4*>(soa + 2 * B);
+            v.GX = reinterpret_cast<const float4*>(soa + (ADJ ? 3 : 0) * B);
+            v.GY = reinterpret_cast<const float4*>(soa + (ADJ ? 4 : 0) * B);
+            v.GZ = reinterpret_cast<const float4*>(soa + (ADJ ? 5 : 0) * B);
+            // the centre cell's stages hold the self pairs only for chunks with sinks
+            // in that cell; other chunks run them on the tracked fast path
+            bool exact = it.has_self && st < nst0;
+            // Sources of ring 2 and beyond are at least one cell away from every
+            // sink of the pencil, and every source is more than one cell away from
+            // the sinks of cells two or more cells from the plane in x: the top hat
+            // (b <= one cell) and the softened branch (eps_s <= one cell) cannot
+            // occur there.
+            const bool far = beg >= it.n_near || !it.near_x;
+            const bool dens = DENS && (!dens_near_only || !far);
+            if (!exact) {
+#pragma unroll
+                for (int s = 0; s < S; ++s) k.sx[s] = k.sy[s] = k.sz[s] = k.sw[s] = 0ull;
+                float trk = kBig;
+                if (far && soft_near_only) {
+                    if constexpr (ADJ) stage_adj_fast<S, false>(v, cnt, k, trk);
+                    else if (dens) stage_fwd_fast<S, DENS, false>(v, cnt, k, trk, b2);
+                    else stage_fwd_fast<S, false, false>(v, cnt, k, trk, b2);
+                } else {
+                    if constexpr (ADJ) stage_adj_fast<S>(v, cnt, k, trk);
+                    else if (dens && !dens_defer) stage_fwd_fast<S, DENS>(v, cnt, k, trk, b2);
+                    else stage_fwd_fast<S, false>(v, cnt, k, trk, b2);
+                    exact = __any_sync(kFull, trk < cf.eps2);
+                    if (exact && lane == 0) atomicAdd(&hdr->stages_rerun, 1ull);  // rare
+                    if constexpr (DENS && !ADJ) {
+                        // a pair closer than b gives a positive term; elsewhere every term is +0
+                        if (dens && dens_defer && !exact && __any_sync(kFull, trk < lo(b2)))
+                            stage_density<S>(v, cnt, k, b2);
+                    }
                 }
             }
-        }
-        if (exact) {
+            if (exact) {
 #pragma unroll
-            for (int s = 0; s < S; ++s) k.sx[s] = k.sy[s] = k.sz[s] = k.sw[s] = 0ull;
-            if constexpr (ADJ) stage_adj_exact<S>(v, cnt, k, cf);
-            else if (dens) stage_fwd_exact<S, DENS>(v, cnt, k, cf, b2);
-            else stage_fwd_exact<S, false>(v, cnt, k, cf, b2);
+                for (int s = 0; s < S; ++s) k.sx[s] = k.sy[s] = k.sz[s] = k.sw[s] = 0ull;
+                if constexpr (ADJ) stage_adj_exact<S>(v, cnt, k, cf);
+                else if (dens) stage_fwd_exact<S, DENS>(v, cnt, k, cf, b2);
+                else stage_fwd_exact<S, false>(v, cnt, k, cf, b2);
+            }
+            if constexpr (W == 1) {
+#pragma unroll
+                for (int s = 0; s < S; ++s) {
+                    k.ax[s] += lo(k.sx[s]) + hi(k.sx[s]);
+                    k.ay[s] += lo(k.sy[s]) + hi(k.sy[s]);
+                    k.az[s] += lo(k.sz[s]) + hi(k.sz[s]);
+                    if constexpr (DENS) k.aw[s] += lo(k.sw[s]) + hi(k.sw[s]);
+                }
+            } else {
+                float* mine = wb.stage_sums + (size_t)w * (NS * S * 32) + lane;
+#pragma unroll
+                for (int s = 0; s < S; ++s) {
+                    mine[(NS * s + 0) * 32] = lo(k.sx[s]) + hi(k.sx[s]);
+                    mine[(NS * s + 1) * 32] = lo(k.sy[s]) + hi(k.sy[s]);
+                    mine[(NS * s + 2) * 32] = lo(k.sz[s]) + hi(k.sz[s]);
+                    if constexpr (DENS) mine[(NS * s + 3) * 32] = lo(k.sw[s]) + hi(k.sw[s]);
+                }
+            }
+            __syncwarp();
         }
+        if constexpr (W > 1) {
+            __syncthreads();
+            const int n = min(W, nst - st0);
+            for (int q = w; q < NS * S; q += W) {
+                float t = wb.totals[q * 32 + lane];
+                for (int j = 0; j < n; ++j) t += wb.stage_sums[((size_t)j * (NS * S) + q) * 32 + lane];
+                wb.totals[q * 32 + lane] = t;
+            }
+            __syncthreads();
+        }
+    }
+    if constexpr (W > 1) {
+        __syncthreads();  // the totals are complete (and cleared where there was no stage)
 #pragma unroll
         for (int s = 0; s < S; ++s) {
-            k.ax[s] += lo(k.sx[s]) + hi(k.sx[s]);
-            k.ay[s] += lo(k.sy[s]) + hi(k.sy[s]);
-            k.az[s] += lo(k.sz[s]) + hi(k.sz[s]);
-            if constexpr (DENS) k.aw[s] += lo(k.sw[s]) + hi(k.sw[s]);
+            k.ax[s] = wb.totals[(NS * s + 0) * 32 + lane];
+            k.ay[s] = wb.totals[(NS * s + 1) * 32 + lane];
+            k.az[s] = wb.totals[(NS * s + 2) * 32 + lane];
+            if constexpr (DENS) k.aw[s] = wb.totals[(NS * s + 3) * 32 + lane];
         }
-        __syncwarp();
     }
 #pragma unroll
     for (int s = 0; s < S; ++s) {
+        if (W > 1 && s % W != w) continue;  // the warps share the sinks' rows
         const int p = it.chunk_begin + s * 32 + lane;
         int at, slot;
         sink_lookup(it, p, &at, &slot);
@@ -731,8 +775,9 @@ __device__ __forceinline__ void run_item(const ItemCtx& it, const Coef& cf, f2 b
 
 // MINB = 2 allows 128 registers per thread (16 resident warps per SM);
 // MINB = 3 caps them at 85 so 24 warps fit (the "lean" variant, for S <= 2).
-template <int SMAX, int B, bool ADJ, int MINB, bool DENS>
-__global__ void __launch_bounds__(256, MINB)
+// NW > 1: a block of NW warps shares every item (run_item).
+template <int SMAX, int B, bool ADJ, int MINB, bool DENS, int NW = 1>
+__global__ void __launch_bounds__(NW > 1 ? 32 * NW : 256, MINB)
 k_force(const BoxDev* __restrict__ boxes, const int* __restrict__ off, const float4* __restrict__ rel,
         const float4* __restrict__ gs, const int4* __restrict__ items, WsHeader* hdr,
         float4* __restrict__ partial, int pstride, int max_nseg)
@@ -753,11 +798,21 @@ k_force(const BoxDev* __restrict__ boxes, const int* __restrict__ off, const flo
 
     const int n_items = *((volatile int*)&hdr->n_items);
     constexpr int CH = 32 * SMAX;
+    wb.stage_sums = reinterpret_cast<float*>(smem + (size_t)NW * W::bytes(max_nseg));
+    wb.totals = wb.stage_sums + (size_t)NW * (DENS ? 4 : 3) * SMAX * 32;
 
     for (;;) {
         int itn = 0;
-        if (lane == 0) itn = atomicAdd(&hdr->queue, 1);
-        itn = __shfl_sync(kFull, itn, 0);
+        if constexpr (NW == 1) {
+            if (lane == 0) itn = atomicAdd(&hdr->queue, 1);
+            itn = __shfl_sync(kFull, itn, 0);
+        } else {
+            __shared__ int next;
+            if (threadIdx.x == 0) next = atomicAdd(&hdr->queue, 1);
+            __syncthreads();
+            itn = next;
+            __syncthreads();  // read before the next one is written
+        }
         if (itn >= n_items) break;
         const int4 item = items[itn];
         const BoxDev& Bx = boxes[item.z];
@@ -838,7 +893,7 @@ k_force(const BoxDev* __restrict__ boxes, const int* __restrict__ off, const flo
         }
         const int S = (n_chunk + 31) >> 5;  // <= SMAX
 #define NF_RUN_ITEM(SS)                                                                                   \
-    run_item<(SMAX >= SS ? SS : 1), B, ADJ, DENS>(it, cf, b2, rel, gs, wb, seg_pre, seg_start, seg_dy, seg_dz, \
+    run_item<(SMAX >= SS ? SS : 1), B, ADJ, DENS, NW>(it, cf, b2, rel, gs, wb, seg_pre, seg_start, seg_dy, seg_dz, \
                                                   partial, pstride, hdr)
         if (SMAX >= 8 && S == 8) NF_RUN_ITEM(8);
         else if (SMAX >= 7 && S == 7) NF_RUN_ITEM(7);
@@ -1029,6 +1084,16 @@ typedef void (*ForceKernel)(const BoxDev*, const int*, const float4*, const floa
 // resident warps per SM.
 bool wants_lean(const ForceTuning& t) { return t.sinks_per_lane <= 2 && t.warps_per_block * t.blocks_per_sm >= 24; }
 
+// Cooperative builds: W warps to an item of four sinks per lane (the built-in
+// shapes' sums), 16 (adjoint: 8) resident warps per SM.
+template <bool ADJ, bool DENS>
+ForceKernel pick_coop(int W)
+{
+    if constexpr (!ADJ)
+        if (W == 8) return k_force<4, 128, ADJ, 2, DENS, 8>;
+    return W == 4 ? k_force<4, 128, ADJ, ADJ ? 2 : 4, DENS, 4> : nullptr;
+}
+
 template <bool ADJ, bool DENS>
 ForceKernel pick_kernel(const ForceTuning& t)
 {
@@ -1063,18 +1128,23 @@ ForceKernel pick_kernel(const ForceTuning& t)
     return nullptr;
 }
 
-ForceKernel pick(bool adjoint, bool density, const ForceTuning& t)
+ForceKernel pick(bool adjoint, bool density, const ForceTuning& t, int coop)
 {
+    if (coop > 1) {
+        if (t.sinks_per_lane != 4 || t.stage != 128) return nullptr;
+        if (adjoint) return pick_coop<true, false>(coop);
+        return density ? pick_coop<false, true>(coop) : pick_coop<false, false>(coop);
+    }
     if (adjoint) return pick_kernel<true, false>(t);
     return density ? pick_kernel<false, true>(t) : pick_kernel<false, false>(t);
 }
 
-size_t force_smem_bytes(bool adjoint, const ForceTuning& t, int max_nseg)
+size_t force_smem_bytes(bool adjoint, const ForceTuning& t, int max_nseg, int warps)
 {
     size_t per = 0;
     if (t.stage == 128) per = adjoint ? WarpSmem<128, true>::bytes(max_nseg) : WarpSmem<128, false>::bytes(max_nseg);
     else per = adjoint ? WarpSmem<64, true>::bytes(max_nseg) : WarpSmem<64, false>::bytes(max_nseg);
-    return per * (size_t)t.warps_per_block;
+    return per * (size_t)warps;
 }
 
 }  // namespace
@@ -1085,19 +1155,6 @@ bool force_tuning_supported(const ForceTuning& t)
     bool b_ok = t.stage == 64 || t.stage == 128;
     bool w_ok = t.warps_per_block == 4 || t.warps_per_block == 8;
     return s_ok && b_ok && w_ok && t.blocks_per_sm >= 0 && t.blocks_per_sm <= 8;
-}
-
-int force_blocks_per_sm(bool adjoint, bool density, const ForceTuning& t, int max_nseg)
-{
-    ForceKernel kfn = pick(adjoint, density, t);
-    if (!kfn) return 0;
-    size_t smem = force_smem_bytes(adjoint, t, max_nseg);
-    if (ensure_smem((const void*)kfn, (int)smem) != cudaSuccess) return 0;
-    int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void*)kfn, t.warps_per_block * 32, smem) !=
-        cudaSuccess)
-        return 0;
-    return nb;
 }
 
 cudaError_t launch_pencils(const BoxDev* boxes, int nboxes, int Ctot, const int* cell_off, int chunk, int stage,
@@ -1135,24 +1192,26 @@ cudaError_t launch_gather_g(const float* g, const int* perm, int Ntot, float4* g
     return cudaGetLastError();
 }
 
-cudaError_t launch_force(bool adjoint, bool density, const ForceTuning& t, const BoxDev* boxes,
+cudaError_t launch_force(bool adjoint, bool density, const ForceTuning& t, int coop, const BoxDev* boxes,
                          const int* cell_off, const float4* rel, const float4* gs, const int4* items,
                          WsHeader* hdr, float4* partial, int pstride, int max_nseg, cudaStream_t s)
 {
-    ForceKernel kfn = pick(adjoint, density, t);
+    ForceKernel kfn = pick(adjoint, density, t, coop);
     if (!kfn) return cudaErrorInvalidValue;
-    size_t smem = force_smem_bytes(adjoint, t, max_nseg);
+    const int warps = coop > 1 ? coop : t.warps_per_block;
+    size_t smem = force_smem_bytes(adjoint, t, max_nseg, warps);
+    if (coop > 1) smem += (size_t)(coop + 1) * (density ? 4 : 3) * t.sinks_per_lane * 32 * sizeof(float);
     cudaError_t e = ensure_smem((const void*)kfn, (int)smem);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     int nb = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void*)kfn, t.warps_per_block * 32, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void*)kfn, warps * 32, smem);
     if (e != cudaSuccess) return e;
     if (nb < 1) return cudaErrorInvalidConfiguration;
-    if (t.blocks_per_sm > 0 && t.blocks_per_sm < nb) nb = t.blocks_per_sm;
-    kfn<<<sms * nb, t.warps_per_block * 32, smem, s>>>(boxes, cell_off, rel, gs, items, hdr, partial, pstride,
+    if (coop <= 1 && t.blocks_per_sm > 0 && t.blocks_per_sm < nb) nb = t.blocks_per_sm;
+    kfn<<<sms * nb, warps * 32, smem, s>>>(boxes, cell_off, rel, gs, items, hdr, partial, pstride,
                                                        max_nseg);
     count_launches(1);
     return cudaGetLastError();

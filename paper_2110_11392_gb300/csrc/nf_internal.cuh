@@ -269,7 +269,9 @@ cudaError_t launch_items(const BoxDev* boxes, int nboxes, int Ctot, const int* c
                          int4* items, WsHeader* hdr, cudaStream_t s);
 cudaError_t launch_gather_g(const float* g, const int* perm, int Ntot, float4* gs,
                             cudaStream_t s);
-cudaError_t launch_force(bool adjoint, bool density, const ForceTuning& t, const BoxDev* boxes,
+// coop: warps that share an item (1, 4 or, forward, 8; above 1 only for four sinks per lane and
+// stages of 128), without effect on the results
+cudaError_t launch_force(bool adjoint, bool density, const ForceTuning& t, int coop, const BoxDev* boxes,
                          const int* cell_off, const float4* rel, const float4* gs,
                          const int4* items, WsHeader* hdr, float4* partial, int pstride,
                          int max_nseg, cudaStream_t s);
@@ -308,6 +310,5 @@ cudaError_t launch_drift(float* pos, const float* vel, int N, const double* dt, 
 cudaError_t launch_timestep(const int* off, const int* perm, const float* vel, const float* acc, int C, long long N,
                             double eta_acc, double eta_h, double hubble, StepScratch* st, double* dt,
                             cudaStream_t s);
-int force_blocks_per_sm(bool adjoint, bool density, const ForceTuning& t, int max_nseg);
 
 }  // namespace nf
