@@ -170,11 +170,18 @@ size_t directed_bytes(int64_t N, int64_t C, int R)
 // next step, so the last bits of the sums decide a run's trajectory, and a run
 // continued with this version keeps it.
 constexpr int64_t kSymMinN = int64_t(1) << 18, kSymMaxN = int64_t(1) << 28;
-bool sym_box(const nf_box& b)
+// A box whose pencils hold too few sinks at mean occupancy for the symmetric
+// kernel's lanes (fill_needed) is not considered: the choice costs two launches.
+bool sym_box(const nf_box& b, bool adjoint)
 {
-    return b.N >= kSymMinN && b.N <= kSymMaxN &&
-           directed_bytes(b.N, (int64_t)b.K * b.K * b.K, b.R) > (size_t)NF_NOALLOC_SCRATCH_BYTES;
+    const int64_t cells = (int64_t)b.K * b.K * b.K;
+    const double sinks = (2.0 * b.R + 1.0) * (double)b.N / (double)cells;
+    const double needed = b.N >= 1500000 ? 160.0 : adjoint ? 180.0 : b.N >= 450000 ? 260.0 : 430.0;
+    return b.N >= kSymMinN && b.N <= kSymMaxN && sinks >= needed &&
+           directed_bytes(b.N, cells, b.R) > (size_t)NF_NOALLOC_SCRATCH_BYTES;
 }
+// Which boxes a plan may give to the symmetric kernel.
+enum class Sym { no, forward, adjoint };
 // Tile groups of a dear pencil: the fewer pencils a warp has, the finer they are
 // cut (clustered 10^6 forward: 8 groups 3.59 ms, 4 3.88, 2 4.07; 200^3: 33.6, 33.4,
 // 33.1, where the combine's 0.94, 0.66, 0.52 ms for the slots weigh more).
@@ -191,10 +198,12 @@ int sym_box_groups(int64_t N)
 // 65536 clustered (3000) 516 -> 374, 131072 clustered (6591) 717 -> 640, 230000 (10125)
 // 938 against 998 with four; adjoint 174 -> 111, 290 -> 234, 373 -> 342, and 602 against
 // 631 with four at 3000 items.
-int coop_warps(int64_t items, bool adjoint)
+// With few stages to an item (R = 1) there is less to share: 265000 particles in 19^3
+// cells (6859 items of 4 stages) take 282 us with one warp and 307 with four.
+int coop_warps(int64_t items, int64_t stages, bool adjoint)
 {
     if (adjoint) return items < 2000 ? 4 : 1;
-    return items < 1000 ? 8 : items < 8000 ? 4 : 1;
+    return items < 1000 ? 8 : items < (stages >= 8 * items ? 8000 : 2500) ? 4 : 1;
 }
 bool same_tuning(const ForceTuning& a, const ForceTuning& b)
 {
@@ -213,7 +222,8 @@ struct Plan {
     int64_t N = 0;       // total particles
     int64_t C = 0;       // total cells
     int64_t max_items = 0;
-    int64_t mean_items = 0;  // work items if every cell held its box's mean occupancy
+    // work items, and their stages in all, if every cell held its box's mean occupancy
+    int64_t mean_items = 0, mean_stages = 0;
     int max_R = 1;
     int max_nseg = 9;
     int nchunks = 0;     // combine chunks
@@ -279,15 +289,15 @@ int make_box(const nf_box& in, bool need_force, BoxDev* out)
     return NF_OK;
 }
 
-// sym: boxes within the symmetric kernel's sizes run there (else all are directed)
-int make_plan(const nf_box* boxes, int nboxes, bool need_force, int chunk_lanes, Plan* p, bool sym = false)
+// sym: boxes within the symmetric kernel's sizes may run there (else all are directed)
+int make_plan(const nf_box* boxes, int nboxes, bool need_force, int chunk_lanes, Plan* p, Sym sym = Sym::no)
 {
     if (!boxes || nboxes < 1) return fail(NF_ERR_ARG, "need at least one box");
     p->nboxes = nboxes;
     p->boxes.resize(nboxes);
     int64_t N = 0, C = 0, items = 0, nchunks = 0, units = 0, planes = 0;
     p->any_sym = false;
-    p->mean_items = 0;
+    p->mean_items = p->mean_stages = 0;
     int max_R = 1;
     for (int b = 0; b < nboxes; ++b) {
         int rc = make_box(boxes[b], need_force, &p->boxes[b]);
@@ -308,14 +318,17 @@ int make_plan(const nf_box* boxes, int nboxes, bool need_force, int chunk_lanes,
         nchunks += (boxes[b].N + kCombineChunk - 1) / kCombineChunk;
         if (need_force) {
             if (d.R > max_R) max_R = d.R;
-            if (sym && sym_box(boxes[b])) {
+            if (sym != Sym::no && sym_box(boxes[b], sym == Sym::adjoint)) {
                 d.sym = 1;
                 d.groups = sym_box_groups(d.N);
                 units += sym_max_units(d.N, cells, d.R, d.groups);
                 p->any_sym = true;
             }
             items += directed_items(d.N, cells, d.R, chunk_lanes);
-            p->mean_items += cells * (((2 * (int64_t)d.R + 1) * d.N / cells + chunk_lanes - 1) / chunk_lanes);
+            const int64_t ns = 2 * (int64_t)d.R + 1;
+            const int64_t mean = cells * ((ns * d.N / cells + chunk_lanes - 1) / chunk_lanes);
+            p->mean_items += mean;
+            p->mean_stages += mean * (1 + ns * ns * d.N / cells / 128);
         }
         if (N >= (int64_t(1) << 31)) return fail(NF_ERR_ARG, "total N must be < 2^31");
         if (C >= (int64_t(1) << 31) - 1) return fail(NF_ERR_ARG, "total cells must be < 2^31");
@@ -369,7 +382,7 @@ int make_plan(const nf_box* boxes, int nboxes, bool need_force, int chunk_lanes,
         p->o_items = take(16 * (size_t)items);
         p->o_gs = take(16 * (size_t)N);
         p->o_partial = take(4 * (size_t)planes);
-        p->o_sym = p->any_sym ? take(sizeof(SymCtl) + 16 * (size_t)nboxes) : 0;
+        p->o_sym = p->any_sym ? take(sizeof(SymCtl) + 24 * (size_t)nboxes) : 0;
         p->o_sym_dims = p->any_sym ? take(8 * (size_t)C) : 0;
         p->o_sym_units = p->any_sym ? take(16 * (size_t)units) : 0;
         p->o_chunk_sums = take(8 * 3 * (size_t)nchunks);
@@ -482,17 +495,20 @@ int run_forces(const Plan& p, bool adjoint, const ForceTuning& t, const float* p
     int4* units = at<int4>(ws, p.o_sym_units);
     int* chunks = at<int>(ws, p.o_chunks);
     unsigned char* bucket_of = at<unsigned char>(ws, p.o_bucket_of);
-    if (p.any_sym) NF_CUDA(cudaMemsetAsync(sym, 0, sizeof(SymCtl) + 16 * (size_t)p.nboxes, s), "clear units");
+    if (p.any_sym) NF_CUDA(cudaMemsetAsync(sym, 0, sizeof(SymCtl) + 24 * (size_t)p.nboxes, s), "clear units");
     NF_CUDA(launch_pencils(boxes, p.nboxes, (int)p.C, off, CH, t.stage, chunks, bucket_count, bucket_of, dims,
                            sym_total, gm, hdr, s),
             "pencils");
-    if (p.any_sym)
+    int4* items = at<int4>(ws, p.o_items);
+    if (p.any_sym) {
         NF_CUDA(launch_sym_units(adjoint, boxes, p.nboxes, (int)p.C, off, dims, sym, sym_total, units, chunks,
-                                 bucket_of, bucket_count, hdr, s),
-                "symmetric work units");
-    NF_CUDA(launch_bucket_scan(bucket_count, hdr, s), "work items");
-    NF_CUDA(launch_items(boxes, p.nboxes, (int)p.C, chunks, bucket_of, bucket_count, at<int4>(ws, p.o_items), hdr, s),
-            "work items");
+                                 bucket_of, bucket_count, items, hdr, s),
+                "work units");
+    } else {
+        NF_CUDA(launch_bucket_scan(bucket_count, hdr, s), "work items");
+        NF_CUDA(launch_items(boxes, p.nboxes, (int)p.C, chunks, bucket_of, bucket_count, items, hdr, s),
+                "work items");
+    }
     float4* gs = at<float4>(ws, p.o_gs);
     if (adjoint) NF_CUDA(launch_gather_g(g, perm, (int)p.N, gs, s), "gather g");
     float4* partial = at<float4>(ws, p.o_partial);
@@ -503,8 +519,8 @@ int run_forces(const Plan& p, bool adjoint, const ForceTuning& t, const float* p
                                  reinterpret_cast<float*>(partial), s),
                 adjoint ? "symmetric adjoint kernel" : "symmetric force kernel");
     // (with nothing on its list where every box is symmetric)
-    const int coop = builtin_tuning(t, adjoint) && !p.any_sym ? coop_warps(p.mean_items, adjoint) : 1;
-    NF_CUDA(launch_force(adjoint, rho != nullptr, t, coop, boxes, off, rel, gs, at<int4>(ws, p.o_items), hdr, partial,
+    const int coop = builtin_tuning(t, adjoint) && !p.any_sym ? coop_warps(p.mean_items, p.mean_stages, adjoint) : 1;
+    NF_CUDA(launch_force(adjoint, rho != nullptr, t, coop, boxes, off, rel, gs, items, hdr, partial,
                          pstride, p.max_nseg, s),
             adjoint ? "adjoint kernel" : "force kernel");
     NF_CUDA(prof_mark(3, s), "profile");
@@ -548,7 +564,8 @@ int forces_entry(const nf_box* boxes, int nboxes, bool adjoint, const float* pos
     int rc = check_tuning(tune, &t, adjoint);
     if (rc) return rc;
     Plan p;
-    rc = make_plan(boxes, nboxes, true, 32 * t.sinks_per_lane, &p, builtin_tuning(t, adjoint));
+    rc = make_plan(boxes, nboxes, true, 32 * t.sinks_per_lane, &p,
+                   !builtin_tuning(t, adjoint) ? Sym::no : adjoint ? Sym::adjoint : Sym::forward);
     if (rc) return rc;
     if (!pos || !out || (adjoint && !g)) return fail(NF_ERR_ARG, "null pointer argument");
     if (rho) {
@@ -610,12 +627,16 @@ namespace nf {
 namespace {
 
 // Workspace of a force call under any tuning: the directed plan with the most
-// items, or the plan with the symmetric kernel's planes.
+// items, or the plan with the symmetric kernel's planes of either direction.
 size_t force_workspace_bytes(const nf_box* boxes, int nboxes)
 {
-    Plan a, b;
-    if (make_plan(boxes, nboxes, true, 32, &a) || make_plan(boxes, nboxes, true, 32, &b, true)) return 0;
-    return a.total > b.total ? a.total : b.total;
+    size_t most = 0;
+    for (Sym sym : {Sym::no, Sym::forward, Sym::adjoint}) {
+        Plan p;
+        if (make_plan(boxes, nboxes, true, 32, &p, sym)) return 0;
+        most = std::max(most, p.total);
+    }
+    return most;
 }
 
 }  // namespace
@@ -1292,7 +1313,8 @@ int nf_forces_total(const float* pos, int64_t N, double box, int K, int R, doubl
     int rc = check_tuning(nullptr, &t);
     if (rc) return rc;
     Plan pn;
-    rc = make_plan(&b, 1, true, 32 * t.sinks_per_lane, &pn, builtin_tuning(t, false));
+    rc = make_plan(&b, 1, true, 32 * t.sinks_per_lane, &pn,
+                   builtin_tuning(t, false) ? Sym::forward : Sym::no);
     if (rc) return rc;
     if (!pos || !acc) return fail(NF_ERR_ARG, "null pointer argument");
     rc = check_ws(pn, ws, ws_bytes);

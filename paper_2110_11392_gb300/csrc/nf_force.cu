@@ -86,7 +86,7 @@ __global__ void k_pencils(const BoxDev* __restrict__ boxes, int nboxes, int Ctot
     for (int gb = blockIdx.x * blockDim.x; gb < Ctot; gb += gridDim.x * blockDim.x) {
         const int g = gb + (int)threadIdx.x;
         int nch = 0, bk = 0, box = -1;
-        unsigned long long scost = 0;
+        unsigned long long scost = 0, dcost = 0;
         if (g < Ctot) {
             const BoxDev& B = boxes[find_box_by_cell(boxes, nboxes, g)];
             const int K = B.K, R = B.R, cb = B.cell_base;
@@ -118,10 +118,12 @@ __global__ void k_pencils(const BoxDev* __restrict__ boxes, int nboxes, int Ctot
                 const int self_chunks = (c_first + occ + CH - 1) / CH - c_first / CH;
                 stages_exact += (unsigned long long)self_chunks * (unsigned long long)st0;
             }
+            unsigned long long lp = 0;
             if (nch) {
                 int rem = n_sink - (nch - 1) * CH;
                 unsigned long long lanes = (unsigned long long)(nch - 1) * CH + 32ull * ((rem + 31) / 32);
-                lane_pairs += lanes * (unsigned long long)n_src;
+                lp = lanes * (unsigned long long)n_src;
+                lane_pairs += lp;
             }
             if (B.sym) {
                 // the symmetric kernel's pencil: the centre cell and half of the plane as sources
@@ -132,6 +134,7 @@ __global__ void k_pencils(const BoxDev* __restrict__ boxes, int nboxes, int Ctot
                                          &st);
                 sym_dims[g] = make_int2(n_sink, n_half);
                 scost = sym_cost(n_sink, n_half, sym_gm);
+                dcost = lp;
                 box = find_box_by_cell(boxes, nboxes, g);
                 chunks[g] = nch;
                 nch = 0;  // on the directed list only if the box turns out directed (k_sym_count)
@@ -139,15 +142,21 @@ __global__ void k_pencils(const BoxDev* __restrict__ boxes, int nboxes, int Ctot
                 chunks[g] = nch;
             }
         }
-        // the symmetric boxes' total costs: one atomic per box per warp
+        // the symmetric boxes' total costs in either kernel: one atomic each per box per warp
         if (sym_total) {
             const unsigned same = __match_any_sync(kFull, box);
-            unsigned long long sum = 0;
+            unsigned long long sum = 0, dsum = 0;
             for (int src = 0; src < 32; ++src) {
-                const unsigned long long v = __shfl_sync(kFull, scost, src);
-                if ((same >> src) & 1u) sum += v;
+                const unsigned long long v = __shfl_sync(kFull, scost, src), d = __shfl_sync(kFull, dcost, src);
+                if ((same >> src) & 1u) {
+                    sum += v;
+                    dsum += d;
+                }
             }
-            if (box >= 0 && (int)(threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(&sym_total[box], sum);
+            if (box >= 0 && (int)(threadIdx.x & 31) == __ffs(same) - 1) {
+                atomicAdd(&sym_total[box], sum);
+                atomicAdd(&sym_total[2 * nboxes + box], dsum);
+            }
         }
         // one atomic per bucket per warp: most cells of a box fall in a few buckets
         const int key = nch ? bk : -1;
@@ -200,8 +209,7 @@ __global__ void k_items(const BoxDev* __restrict__ boxes, int nboxes, int Ctot,
     const int lane = threadIdx.x & 31;
     for (int gb = blockIdx.x * blockDim.x; gb < Ctot; gb += gridDim.x * blockDim.x) {
         const int g = gb + (int)threadIdx.x;
-        const int box = g < Ctot ? find_box_by_cell(boxes, nboxes, g) : 0;
-        const int nch = g < Ctot && !boxes[box].sym ? chunks[g] : 0;
+        const int nch = g < Ctot ? chunks[g] : 0;
         const int bk = nch ? (int)bucket_of[g] : -1;
         // one atomic per bucket per warp; each lane's chunks follow those of the
         // lanes below it in the same bucket (the order of items within a bucket
@@ -220,7 +228,8 @@ __global__ void k_items(const BoxDev* __restrict__ boxes, int nboxes, int Ctot,
         if (nch && lane == leader) base = atomicAdd(&cursor[bk], tot);
         base = __shfl_sync(kFull, base, leader) + pre;
         if (nch) {
-            for (int q = 0; q < nch; ++q) items[base + q] = make_int4(g, q, box, 0);
+            const int b = find_box_by_cell(boxes, nboxes, g);
+            for (int q = 0; q < nch; ++q) items[base + q] = make_int4(g, q, b, 0);
         }
     }
 }

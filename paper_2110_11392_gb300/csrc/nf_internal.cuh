@@ -61,7 +61,7 @@ struct BoxDev {
     // is closer than b (small b); 0: it is fused into every stage that can hold one
     int dens_defer;
     // symmetric pair kernel (nf_sym.cu): 1 if it may run this box (cleared on the device where the
-    // directed one is the better, k_sym_choose); source-tile groups of a pencil
+    // directed one is the better, k_sym_scan); source-tile groups of a pencil
     int sym;
     int groups;
     // first float of the box's planes of partial sums (symmetric)
@@ -257,7 +257,7 @@ struct ForceTuning {
 };
 
 // sym_dims, sym_total: of the boxes with .sym set, every pencil's (sinks, half-plane
-// sources) and the box's total cost (null when no box is symmetric); their chunks
+// sources) and the box's totals (null when no box is symmetric); their chunks
 // are counted later, if the box turns out to be directed (launch_sym_units)
 cudaError_t launch_pencils(const BoxDev* boxes, int nboxes, int Ctot, const int* cell_off,
                            int chunk, int stage, int* chunks, unsigned* bucket_count,
@@ -289,11 +289,13 @@ bool force_tuning_supported(const ForceTuning& t);
 int sym_slots(int R, int groups);
 int sym_gmax(bool adjoint);  // largest groups of a chunk
 long long sym_max_units(long long N, long long C, int R, int groups);
-// total: [2 nboxes], the boxes' costs and (written here) the costs of their dear pencils.
-// Clears .sym of the boxes that run better directed and adds their chunks to bucket_count.
+// total: [3 nboxes], the boxes' costs, the costs of their dear pencils (written here), and
+// the directed kernel's lane pairs.
+// Clears .sym of the boxes that run better directed; writes both lists (bucket_count holds
+// the other boxes' chunks).
 cudaError_t launch_sym_units(bool adjoint, BoxDev* boxes, int nboxes, int Ctot, const int* cell_off,
                              const int2* dims, SymCtl* ctl, unsigned long long* total, int4* units,
-                             const int* chunks, const unsigned char* bucket_of, unsigned* bucket_count,
+                             const int* chunks, const unsigned char* bucket_of, unsigned* bucket_count, int4* items,
                              WsHeader* hdr, cudaStream_t s);
 cudaError_t launch_sym_force(bool adjoint, bool density, const BoxDev* boxes, const int* cell_off, const float4* rel,
                              const float4* gs, const int4* units, SymCtl* ctl, WsHeader* hdr, float* planes,

@@ -34,8 +34,8 @@
 // than one warp's share of the box, the sinks' half and the sources' half of
 // the work become one-sided units per chunk (22 operations a pair instead of
 // 14, any number of warps).  A box with much of its work in such pencils is left
-// to the directed kernel (k_sym_choose, on the device: the counts are not known
-// on the host).
+// to the directed kernel (box_is_sym, on the device: the counts are not known on
+// the host).
 //
 // Softening and the density follow nf_force.cu: tiles that can hold a pair
 // closer than a cell track the smallest r^2 and are run again on the exact
@@ -76,7 +76,7 @@ constexpr int sym_warps(bool adj) { return 152 * kWarps * (adj ? kBlocksAdj : kB
 // 1.19 at a share of 0.26, 1.07 at 0.35, 1.05 at 0.51, 0.92 at 0.57, 0.78 at 0.66;
 // adjoint 1.36 at 0.01, 0.92 at 0.085 (3e5 particles), 1.04 at 0.09 (9e5), 0.74 at
 // 0.15 (3e5), 0.96 at 0.24.
-constexpr double dear_share(bool adj) { return adj ? 0.08 : 0.5; }
+__host__ __device__ constexpr double dear_share(bool adj) { return adj ? 0.08 : 0.5; }
 
 // Units of one pencil, by its cost against a warp's share of the box: one unit
 // for a light pencil (at most half a share), `groups` units for a dearer one,
@@ -136,30 +136,55 @@ __global__ void k_sym_dear(const BoxDev* __restrict__ boxes, int nboxes, int Cto
     }
 }
 
-// Boxes in which dear pencils hold much of the work run directed.
-__global__ void k_sym_choose(BoxDev* boxes, int nboxes, const unsigned long long* __restrict__ total, double most)
+// Boxes in which dear pencils hold much of the work run directed, and those whose
+// pencils fill the symmetric kernel's lanes badly: few sinks to a pencil (padded to
+// 64; the directed kernel pads to 32) or few sources to a half plane.  fill is the
+// directed kernel's lane pairs over twice the symmetric kernel's, the latter with
+// what a step costs beside its groups (28 and 10 cycles, sym_cost); the fewer
+// particles, the more its longer work list and combine weigh.  Measured over N =
+// 2.65e5 .. 6e6, 40 .. 90 particles per cell, R = 1 .. 3, uniform and clustered, the
+// directed call's time over the symmetric one's: forward N = 6e6 0.98 at a fill of
+// 0.728, 1.14 at 0.795; 2.5e6 1.00 at 0.743, 1.08 at 0.785; 1.2e6 0.94 at 0.728, 1.03
+// at 0.801, 1.11 at 0.814; 4e5 0.98 at 0.768, 1.04 at 0.797, 1.10 at 0.815 (and with
+// the density, which takes the forward's kernel, 0.98 at 0.801, 1.04 at 0.814; 0.95 at
+// 0.797, 1.01 at 0.815); adjoint 7e5 0.99 at 0.747, 1.05 at 0.763; 4e5 0.97 at 0.777,
+// 1.14 at 0.795.  R = 1 boxes of 20 to 60 particles per cell stay directed by this.
+__device__ __forceinline__ double fill_needed(int N, bool adj)
 {
-    for (int b = threadIdx.x; b < nboxes; b += blockDim.x)
-        if (boxes[b].sym && (double)total[nboxes + b] > most * (double)total[b]) boxes[b].sym = 0;
+    if (adj) return N < 450000 ? 0.78 : 0.75;
+    return N < 450000 ? 0.82 : N < 1500000 ? 0.805 : 0.775;
+}
+__device__ __forceinline__ bool box_is_sym(const BoxDev* boxes, int nboxes, const unsigned long long* total, int b,
+                                           bool adjoint)
+{
+    if (!boxes[b].sym) return false;
+    const double cost = (double)total[b];
+    const double fill = (double)total[2 * nboxes + b] * 28.0 / (128.0 * cost);
+    return (double)total[nboxes + b] <= dear_share(adjoint) * cost && fill >= fill_needed(boxes[b].N, adjoint);
 }
 
+// Counts the boxes' units, or the chunks of those that turn out directed.
 __global__ void k_sym_count(const BoxDev* __restrict__ boxes, int nboxes, int Ctot, const int* __restrict__ off,
                             const int2* __restrict__ dims, const unsigned long long* __restrict__ total, int GM,
-                            int warps, const int* __restrict__ chunks, const unsigned char* __restrict__ bucket_of,
-                            unsigned* __restrict__ sym_count, unsigned* __restrict__ dir_count)
+                            int warps, bool adjoint, const int* __restrict__ chunks,
+                            const unsigned char* __restrict__ bucket_of, unsigned* __restrict__ sym_count,
+                            unsigned* __restrict__ dir_count)
 {
+    __shared__ bool one_sym;
+    if (threadIdx.x == 0) one_sym = nboxes == 1 && box_is_sym(boxes, nboxes, total, 0, adjoint);
+    __syncthreads();
     for (int gb = blockIdx.x * blockDim.x; gb < Ctot; gb += gridDim.x * blockDim.x) {
         const int c = gb + (int)threadIdx.x;
         int n = 0, bk = -1;  // bucket, + kBuckets on the directed list
         if (c < Ctot) {
             const int b = find_box_by_cell(boxes, nboxes, c);
-            if (boxes[b].sym) {
+            if (nboxes == 1 ? one_sym : box_is_sym(boxes, nboxes, total, b, adjoint)) {
                 const int2 d = dims[c];
                 const UnitCount u =
                     count_units(d.x, d.y, off[c + 1] - off[c], boxes[b].groups, GM, (double)total[b] / warps);
                 n = u.units;
                 if (n) bk = u.bucket;
-            } else if (total[b]) {  // a box that was a candidate: its chunks are not counted yet
+            } else if (boxes[b].sym) {  // a candidate: its chunks are not counted yet
                 n = chunks[c];
                 if (n) bk = kBuckets + (int)bucket_of[c];
             }
@@ -171,37 +196,46 @@ __global__ void k_sym_count(const BoxDev* __restrict__ boxes, int nboxes, int Ct
     }
 }
 
-__global__ void k_sym_scan(SymCtl* ctl, WsHeader* hdr)
+// Exclusive scans of both lists' buckets; the boxes' kernels for good.
+__global__ void k_sym_scan(BoxDev* boxes, int nboxes, const unsigned long long* __restrict__ total, bool adjoint,
+                           SymCtl* ctl, unsigned* dir_count, WsHeader* hdr)
 {
-    __shared__ unsigned v[kBuckets];
-    const int t = threadIdx.x;
-    v[t] = ctl->bucket[t];
+    __shared__ unsigned v[2][kBuckets];
+    const int t = threadIdx.x & (kBuckets - 1), list = threadIdx.x / kBuckets;
+    unsigned* count = list ? dir_count : ctl->bucket;
+    v[list][t] = count[t];
     __syncthreads();
     if (t == 0) {
         unsigned run = 0;
         for (int b = 0; b < kBuckets; ++b) {
-            const unsigned c = v[b];
-            v[b] = run;
+            const unsigned c = v[list][b];
+            v[list][b] = run;
             run += c;
         }
-        ctl->n_units = (int)run;
-        hdr->sym_units = (int)run;
+        if (list) hdr->n_items = (int)run;
+        else hdr->sym_units = ctl->n_units = (int)run;
     }
     __syncthreads();
-    ctl->bucket[t] = v[t];
+    count[t] = v[list][t];
+    for (int b = threadIdx.x; b < nboxes; b += blockDim.x)
+        boxes[b].sym = box_is_sym(boxes, nboxes, total, b, adjoint);
 }
 
 // Unit types (item .w)
 constexpr int kUnitSym = 0, kUnitSinks = 1, kUnitSources = 2;
 
+// Writes both lists bucket by bucket (as k_items): symmetric units, and the directed
+// items of the other boxes.
 __global__ void k_sym_units(const BoxDev* __restrict__ boxes, int nboxes, int Ctot, const int* __restrict__ off,
-                            const int2* __restrict__ dims, const unsigned long long* __restrict__ total, int GM, int warps,
-                            unsigned* __restrict__ cursor, int4* __restrict__ units)
+                            const int2* __restrict__ dims, const unsigned long long* __restrict__ total, int GM,
+                            int warps, const int* __restrict__ chunks, const unsigned char* __restrict__ bucket_of,
+                            unsigned* __restrict__ sym_cursor, unsigned* __restrict__ dir_cursor,
+                            int4* __restrict__ units, int4* __restrict__ items)
 {
     const int lane = threadIdx.x & 31;
     for (int gb = blockIdx.x * blockDim.x; gb < Ctot; gb += gridDim.x * blockDim.x) {
         const int c = gb + (int)threadIdx.x;
-        int bk = -1, b = 0, groups = 1;
+        int bk = -1, b = 0, groups = 1, n = 0;
         UnitCount u = {};
         if (c < Ctot) {
             b = find_box_by_cell(boxes, nboxes, c);
@@ -209,25 +243,32 @@ __global__ void k_sym_units(const BoxDev* __restrict__ boxes, int nboxes, int Ct
                 const int2 d = dims[c];
                 groups = boxes[b].groups;
                 u = count_units(d.x, d.y, off[c + 1] - off[c], groups, GM, (double)total[b] / warps);
-                if (u.units) bk = u.bucket;
+                n = u.units;
+                if (n) bk = u.bucket;
+            } else {
+                n = chunks[c];
+                if (n) bk = kBuckets + (int)bucket_of[c];
             }
         }
         const unsigned peers = __match_any_sync(kFull, bk);
         const int leader = __ffs(peers) - 1;
         unsigned pre = 0, tot = 0;
         for (int src = 0; src < 32; ++src) {
-            const unsigned v = __shfl_sync(kFull, (unsigned)u.units, src);
+            const unsigned v = __shfl_sync(kFull, (unsigned)n, src);
             if ((peers >> src) & 1u) {
                 tot += v;
                 if (src < lane) pre += v;
             }
         }
         unsigned base = 0;
-        if (bk >= 0 && lane == leader) base = atomicAdd(&cursor[bk], tot);
+        if (bk >= 0 && lane == leader)
+            base = atomicAdd(bk < kBuckets ? &sym_cursor[bk] : &dir_cursor[bk - kBuckets], tot);
         base = __shfl_sync(kFull, base, leader) + pre;
         if (bk < 0) continue;  // no warp-wide operation follows in this iteration
-        if (!u.heavy) {
-            for (int q = 0; q < u.units; ++q) units[base + q] = make_int4(c, u.light ? -1 : q, b, kUnitSym);
+        if (bk >= kBuckets) {
+            for (int q = 0; q < n; ++q) items[base + q] = make_int4(c, q, b, 0);
+        } else if (!u.heavy) {
+            for (int q = 0; q < n; ++q) units[base + q] = make_int4(c, u.light ? -1 : q, b, kUnitSym);
         } else {
             unsigned at = base;
             for (int q = 0; q < u.nch * groups; ++q) units[at++] = make_int4(c, q, b, kUnitSinks);
@@ -241,12 +282,11 @@ __global__ void k_sym_units(const BoxDev* __restrict__ boxes, int nboxes, int Ct
 // ---------------------------------------------------------------------------
 
 // Resident particles of a lane: two per group, one in each half.
-template <int G, bool ADJ, bool DENS>
+template <int G, bool ADJ>
 struct Residents {
     f2 nx[G], ny[G], nz[G];                                      // -position
     f2 ngx[ADJ ? G : 1], ngy[ADJ ? G : 1], ngz[ADJ ? G : 1];     // -g
     f2 sx[G], sy[G], sz[G];                                      // sums of the current tile
-    f2 sw[DENS ? G : 1];
 };
 
 // Reaction sums of the source a lane holds in this step (they travel with it):
@@ -269,10 +309,17 @@ __device__ __forceinline__ f2 shfl2(f2 v, int src)
     return pk(__shfl_sync(kFull, lo(v), src), __shfl_sync(kFull, hi(v), src));
 }
 
-// One tile, f = r^-3 for every pair.  FORCE off: the density alone.
-template <int G, bool REACT, bool TRK, bool DENS, bool FORCE, bool RD>
-__device__ __forceinline__ void tile_fwd(const Tile& v, Residents<G, false, RD>& k, Reaction& a, float& trk, f2 b2)
+// One tile, f = r^-3 for every pair.  FORCE off: the density alone.  The density's
+// sums live only in the loops that take it (few tiles) and join the running ones in
+// shared memory at once: totw[s * stride], stride TS.
+template <int G, bool REACT, bool TRK, bool DENS, bool FORCE, int TS>
+__device__ __forceinline__ void tile_fwd(const Tile& v, Residents<G, false>& k, Reaction& a, float& trk, f2 b2,
+                                         f2* totw)
 {
+    f2 sw[DENS ? G : 1];
+    if constexpr (DENS)
+#pragma unroll
+        for (int s = 0; s < G; ++s) sw[s] = 0ull;
     const f2 tiny = pk(kTiny, kTiny);
     const int next = (threadIdx.x + 1) & 31;
 #pragma unroll 1
@@ -288,7 +335,7 @@ __device__ __forceinline__ void tile_fwd(const Tile& v, Residents<G, false, RD>&
             if constexpr (TRK) trk = track_min(trk, r2);
             if constexpr (DENS) {
                 const f2 w = tophat2(r2, b2);
-                k.sw[s] = add2(k.sw[s], w);
+                sw[s] = add2(sw[s], w);
                 if constexpr (REACT) a.w = add2(a.w, w);
             }
             if constexpr (FORCE) {
@@ -313,6 +360,9 @@ __device__ __forceinline__ void tile_fwd(const Tile& v, Residents<G, false, RD>&
             if constexpr (DENS) a.w = shfl2(a.w, next);
         }
     }
+    if constexpr (DENS)
+#pragma unroll
+        for (int s = 0; s < G; ++s) totw[s * TS] = add2(totw[s * TS], sw[s]);
 }
 
 // Keeps the halves of v whose bits are set.
@@ -324,10 +374,14 @@ __device__ __forceinline__ f2 keep2(f2 v, unsigned bits)
 // One tile, f = min(poly(r), r^-3) (Eq. (spline) with the min hand-off).  Bit
 // 2s + h of ms0 / mr0: the resident s, h receives the force / acts on the source,
 // for the tile's first n_self sources.
-template <int G, bool REACT, bool DENS, bool RD>
-__device__ __forceinline__ void tile_fwd_exact(const Tile& v, Residents<G, false, RD>& k, Reaction& a, const Coef& cf,
-                                               f2 b2, unsigned ms0, unsigned mr0, int n_self)
+template <int G, bool REACT, bool DENS, int TS>
+__device__ __forceinline__ void tile_fwd_exact(const Tile& v, Residents<G, false>& k, Reaction& a, const Coef& cf,
+                                               f2 b2, unsigned ms0, unsigned mr0, int n_self, f2* totw)
 {
+    f2 sw[DENS ? G : 1];
+    if constexpr (DENS)
+#pragma unroll
+        for (int s = 0; s < G; ++s) sw[s] = 0ull;
     const f2 tiny = pk(kTiny, kTiny);
     const f2 c0 = pk(cf.c0, cf.c0), c1 = pk(cf.c1, cf.c1), c2 = pk(cf.c2, cf.c2);
     const int next = (threadIdx.x + 1) & 31;
@@ -346,7 +400,7 @@ __device__ __forceinline__ void tile_fwd_exact(const Tile& v, Residents<G, false
             r2 = fma2(dz, dz, r2);
             if constexpr (DENS) {
                 const f2 w = tophat2(r2, b2);
-                k.sw[s] = add2(k.sw[s], keep2(w, ms >> (2 * s)));
+                sw[s] = add2(sw[s], keep2(w, ms >> (2 * s)));
                 if constexpr (REACT) a.w = add2(a.w, keep2(w, mr >> (2 * s)));
             }
             const f2 ri = rsqrt2(r2);
@@ -371,11 +425,14 @@ __device__ __forceinline__ void tile_fwd_exact(const Tile& v, Residents<G, false
             if constexpr (DENS) a.w = shfl2(a.w, next);
         }
     }
+    if constexpr (DENS)
+#pragma unroll
+        for (int s = 0; s < G; ++s) totw[s * TS] = add2(totw[s * TS], sw[s]);
 }
 
 // Adjoint, one tile: J v = r^-3 (v - 3 r^-2 (d.v) d), v = g_j - g_i.
 template <int G, bool REACT, bool TRK>
-__device__ __forceinline__ void tile_adj(const Tile& v, Residents<G, true, false>& k, Reaction& a, float& trk)
+__device__ __forceinline__ void tile_adj(const Tile& v, Residents<G, true>& k, Reaction& a, float& trk)
 {
     const f2 tiny = pk(kTiny, kTiny), m3 = pk(-3.0f, -3.0f);
     const int next = (threadIdx.x + 1) & 31;
@@ -418,7 +475,7 @@ __device__ __forceinline__ void tile_adj(const Tile& v, Residents<G, true, false
 
 // Adjoint, one tile, exact: the softened branch selected per pair (as nf_force.cu's stage_adj_exact).
 template <int G, bool REACT>
-__device__ __forceinline__ void tile_adj_exact(const Tile& v, Residents<G, true, false>& k, Reaction& a,
+__device__ __forceinline__ void tile_adj_exact(const Tile& v, Residents<G, true>& k, Reaction& a,
                                                const Coef& cf, unsigned ms0, unsigned mr0, int n_self)
 {
     const f2 tiny = pk(kTiny, kTiny), m3 = pk(-3.0f, -3.0f);
@@ -561,7 +618,7 @@ __device__ __forceinline__ void run_pass(const Pass& ps, int R, const Coef& cf, 
     };
     if (ps.t0 < ps.t1) issue(ps.t0);
 
-    Residents<G, ADJ, DENS> k;
+    Residents<G, ADJ> k;
     unsigned ms = 0, mr = 0;
     {
         int q = 0;
@@ -596,6 +653,11 @@ __device__ __forceinline__ void run_pass(const Pass& ps, int R, const Coef& cf, 
     const bool soft_near_only = cf.eps2 <= 1.0f;  // eps_s <= one cell width
     const bool dens_defer = DENS && cf.dens_defer != 0 && dens_near_only;
     const Tile tv = {xy + lane, zz + lane, gxy + lane, gz + lane};
+    constexpr int TS = L::NS * 32;
+    f2* totw = tot + (DENS ? 96 : 0);
+    if constexpr (DENS)
+#pragma unroll
+        for (int s = 0; s < G; ++s) totw[s * TS] = 0ull;
 
     for (int t = ps.t0; t < ps.t1; ++t) {
         const int my_at = at, my_seg = cur;
@@ -627,16 +689,17 @@ __device__ __forceinline__ void run_pass(const Pass& ps, int R, const Coef& cf, 
         const bool far = 32 * t >= ps.far_from;
         bool exact = ps.exact || n_self > 0;
         const bool dens = DENS && (!dens_near_only || !far);
+        bool fused = false;  // the density is taken in the fast loop
         const bool plain = !exact && far && soft_near_only;  // no pair of this tile can need the exact path
         Reaction a;
         auto clear = [&]() {
 #pragma unroll
             for (int s = 0; s < G; ++s) {
                 k.sx[s] = k.sy[s] = k.sz[s] = 0ull;
-                if constexpr (DENS) k.sw[s] = 0ull;
             }
-            a.x = a.y = a.z = a.w = 0ull;
+            a.x = a.y = a.z = 0ull;
         };
+        a.w = 0ull;
         clear();
         if (!exact) {
             float trk = kBig;
@@ -644,25 +707,25 @@ __device__ __forceinline__ void run_pass(const Pass& ps, int R, const Coef& cf, 
                 if constexpr (ADJ) tile_adj<G, REACT, false>(tv, k, a, trk);
                 else {
                     if constexpr (DENS) {
-                        if (dens) tile_fwd<G, REACT, false, true, true, DENS>(tv, k, a, trk, b2);
+                        if (dens) tile_fwd<G, REACT, false, true, true, TS>(tv, k, a, trk, b2, totw);
                     }
-                    if (!dens) tile_fwd<G, REACT, false, false, true, DENS>(tv, k, a, trk, b2);
+                    if (!dens) tile_fwd<G, REACT, false, false, true, TS>(tv, k, a, trk, b2, totw);
                 }
             } else {
                 if constexpr (ADJ) tile_adj<G, REACT, true>(tv, k, a, trk);
                 else {
-                    const bool fused = dens && !dens_defer;
+                    fused = dens && !dens_defer;
                     if constexpr (DENS) {
-                        if (fused) tile_fwd<G, REACT, true, true, true, DENS>(tv, k, a, trk, b2);
+                        if (fused) tile_fwd<G, REACT, true, true, true, TS>(tv, k, a, trk, b2, totw);
                     }
-                    if (!fused) tile_fwd<G, REACT, true, false, true, DENS>(tv, k, a, trk, b2);
+                    if (!fused) tile_fwd<G, REACT, true, false, true, TS>(tv, k, a, trk, b2, totw);
                 }
                 exact = __any_sync(kFull, trk < cf.eps2);
                 if (exact && lane == 0) atomicAdd(&hdr->stages_rerun, 1ull);  // rare
                 if constexpr (DENS && !ADJ) {
                     // a pair closer than b gives a positive term; elsewhere every term is +0
                     if (dens && dens_defer && !exact && __any_sync(kFull, trk < lo(b2)))
-                        tile_fwd<G, REACT, false, true, false, DENS>(tv, k, a, trk, b2);
+                        tile_fwd<G, REACT, false, true, false, TS>(tv, k, a, trk, b2, totw);
                 }
                 if (exact) clear();
             }
@@ -671,9 +734,10 @@ __device__ __forceinline__ void run_pass(const Pass& ps, int R, const Coef& cf, 
             if constexpr (ADJ) tile_adj_exact<G, REACT>(tv, k, a, cf, ms, mr, n_self);
             else {
                 if constexpr (DENS) {
-                    if (dens) tile_fwd_exact<G, REACT, true, DENS>(tv, k, a, cf, b2, ms, mr, n_self);
+                    if (dens && !fused) tile_fwd_exact<G, REACT, true, TS>(tv, k, a, cf, b2, ms, mr, n_self, totw);
                 }
-                if (!dens) tile_fwd_exact<G, REACT, false, DENS>(tv, k, a, cf, b2, ms, mr, n_self);
+                // (a re-run keeps the density that the fused loop has taken: the term is the same)
+                if (!dens || fused) tile_fwd_exact<G, REACT, false, TS>(tv, k, a, cf, b2, ms, mr, n_self, totw);
             }
         }
         // the tile's sums join the running ones (chains of at most 32 sources)
@@ -684,12 +748,10 @@ __device__ __forceinline__ void run_pass(const Pass& ps, int R, const Coef& cf, 
                 p[0] = k.sx[s];
                 p[32] = k.sy[s];
                 p[64] = k.sz[s];
-                if constexpr (DENS) p[96] = k.sw[s];
             } else {
                 p[0] = add2(p[0], k.sx[s]);
                 p[32] = add2(p[32], k.sy[s]);
                 p[64] = add2(p[64], k.sz[s]);
-                if constexpr (DENS) p[96] = add2(p[96], k.sw[s]);
             }
         }
         if constexpr (REACT) {
@@ -724,7 +786,7 @@ __device__ __forceinline__ void run_pass(const Pass& ps, int R, const Coef& cf, 
             const f2* p = tot + (size_t)s * L::NS * 32;
             const bool any = ps.t0 < ps.t1;
             const f2 x = any ? p[0] : 0ull, y = any ? p[32] : 0ull, z = any ? p[64] : 0ull;
-            const f2 w = DENS && any ? p[DENS ? 96 : 0] : 0ull;
+            const f2 w = DENS ? p[DENS ? 96 : 0] : 0ull;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int pos = ps.r0 + (2 * s + h) * 32 + lane;
@@ -954,17 +1016,17 @@ long long sym_max_units(long long N, long long C, int R, int groups)
 
 cudaError_t launch_sym_units(bool adjoint, BoxDev* boxes, int nboxes, int Ctot, const int* cell_off,
                              const int2* dims, SymCtl* ctl, unsigned long long* total, int4* units,
-                             const int* chunks, const unsigned char* bucket_of, unsigned* bucket_count,
+                             const int* chunks, const unsigned char* bucket_of, unsigned* bucket_count, int4* items,
                              WsHeader* hdr, cudaStream_t s)
 {
     const int grid = grid_for(Ctot, 256), warps = sym_warps(adjoint), GM = sym_groups_max(adjoint);
     k_sym_dear<<<grid, 256, 0, s>>>(boxes, nboxes, Ctot, cell_off, dims, total, GM, warps);
-    k_sym_choose<<<1, 256, 0, s>>>(boxes, nboxes, total, dear_share(adjoint));
-    k_sym_count<<<grid, 256, 0, s>>>(boxes, nboxes, Ctot, cell_off, dims, total, GM, warps, chunks, bucket_of,
-                                     ctl->bucket, bucket_count);
-    k_sym_scan<<<1, kBuckets, 0, s>>>(ctl, hdr);
-    k_sym_units<<<grid, 256, 0, s>>>(boxes, nboxes, Ctot, cell_off, dims, total, GM, warps, ctl->bucket, units);
-    count_launches(5);
+    k_sym_count<<<grid, 256, 0, s>>>(boxes, nboxes, Ctot, cell_off, dims, total, GM, warps, adjoint, chunks,
+                                     bucket_of, ctl->bucket, bucket_count);
+    k_sym_scan<<<1, 2 * kBuckets, 0, s>>>(boxes, nboxes, total, adjoint, ctl, bucket_count, hdr);
+    k_sym_units<<<grid, 256, 0, s>>>(boxes, nboxes, Ctot, cell_off, dims, total, GM, warps, chunks, bucket_of,
+                                     ctl->bucket, bucket_count, units, items);
+    count_launches(4);
     return cudaGetLastError();
 }
 
