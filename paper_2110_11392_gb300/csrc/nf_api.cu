@@ -420,7 +420,6 @@ int check_tuning(const nf_tuning* t, ForceTuning* out, bool adjoint = false)
         if (e__ != cudaSuccess) return cuda_fail(e__, where); \
     } while (0)
 
-// Clears the header, uploads the box table, bins every particle.
 // Debug mode: check every guard block of the workspace at the end of a call.
 int finish_call(void* ws, cudaStream_t s)
 {
@@ -431,39 +430,58 @@ int finish_call(void* ws, cudaStream_t s)
     return NF_OK;
 }
 
-// Clears the status header of a workspace and, in debug mode, fills its guard
-// blocks and records them in the header (every call that later runs
-// finish_call on the workspace starts with this).
-int init_ws(const Plan& p, void* ws, cudaStream_t s)
+// Debug mode: fills the workspace's guard blocks and records them in the header.
+int setup_guards(const Plan& p, void* ws, cudaStream_t s)
 {
-    NF_CUDA(cudaMemsetAsync(at<WsHeader>(ws, 0), 0, sizeof(WsHeader), s), "clear header");
-    if (g_debug && !p.guards.empty()) {
-        GuardList gl;
-        std::memset(&gl, 0, sizeof gl);
-        gl.count = (int)std::min<size_t>(p.guards.size(), 24);
-        for (int i = 0; i < gl.count; ++i) gl.off[i] = (long long)p.guards[i];
-        k_guard_setup<<<gl.count, 64, 0, s>>>(ws, gl);
-        count_launches(1);
-        NF_CUDA(cudaGetLastError(), "guard setup");
-    }
+    if (!g_debug || p.guards.empty()) return NF_OK;
+    GuardList gl;
+    std::memset(&gl, 0, sizeof gl);
+    gl.count = (int)std::min<size_t>(p.guards.size(), 24);
+    for (int i = 0; i < gl.count; ++i) gl.off[i] = (long long)p.guards[i];
+    k_guard_setup<<<gl.count, 64, 0, s>>>(ws, gl);
+    count_launches(1);
+    NF_CUDA(cudaGetLastError(), "guard setup");
     return NF_OK;
 }
 
+// Clears the status header of a workspace whose binning is not run (every call that
+// later runs finish_call on a workspace starts with this or with run_binning).
+int init_ws(const Plan& p, void* ws, cudaStream_t s)
+{
+    NF_CUDA(cudaMemsetAsync(at<WsHeader>(ws, 0), 0, sizeof(WsHeader), s), "clear header");
+    return setup_guards(p, ws, s);
+}
+
+// Clears the header (and the work list's counters), uploads the box table, bins
+// every particle.
 int run_binning(const Plan& p, const float* pos, void* ws, int32_t* cell_off, float4* rel, int32_t* perm,
-                cudaStream_t s)
+                cudaStream_t s, bool force = false)
 {
     WsHeader* hdr = at<WsHeader>(ws, 0);
     BoxDev* boxes = at<BoxDev>(ws, p.o_boxes);
-    int rc = init_ws(p, ws, s);
-    if (rc) return rc;
+    ClearList clear;
+    std::memset(&clear, 0, sizeof clear);
+    clear.at[0] = reinterpret_cast<unsigned*>(hdr);
+    clear.words[0] = sizeof(WsHeader) / 4;
+    if (force) {
+        clear.at[1] = at<unsigned>(ws, p.o_bucket_count);
+        clear.words[1] = kBuckets;
+        if (p.any_sym) {
+            clear.at[2] = at<unsigned>(ws, p.o_sym);
+            clear.words[2] = (int)(sizeof(SymCtl) / 4) + 6 * p.nboxes;
+        }
+    }
     for (int first = 0; first < p.nboxes; first += kMaxBoxesPerFill) {
         BoxFill f;
         std::memset(&f, 0, sizeof f);
         f.first = first;
         f.count = std::min(kMaxBoxesPerFill, p.nboxes - first);
         for (int q = 0; q < f.count; ++q) f.b[q] = p.boxes[first + q];
-        NF_CUDA(launch_fill_boxes(f, boxes, s), "box table");
+        NF_CUDA(launch_fill_boxes(f, boxes, clear, s), "box table");
+        std::memset(&clear, 0, sizeof clear);
     }
+    const int rc = setup_guards(p, ws, s);
+    if (rc) return rc;
     bool pow2 = true;
     for (const BoxDev& b : p.boxes) pow2 = pow2 && b.kl_pow2 != 0.0f;
     NF_CUDA(run_sort(p.sp, pos, (int)p.N, (int)p.C, boxes, p.nboxes, at<void>(ws, p.o_sort),
@@ -482,11 +500,10 @@ int run_forces(const Plan& p, bool adjoint, const ForceTuning& t, const float* p
     float4* rel = at<float4>(ws, p.o_rel);
     int32_t* perm = at<int32_t>(ws, p.o_perm);
     NF_CUDA(prof_mark(0, s), "profile");
-    int rc = run_binning(p, pos, ws, off, rel, perm, s);
+    int rc = run_binning(p, pos, ws, off, rel, perm, s, true);
     if (rc) return rc;
     NF_CUDA(prof_mark(1, s), "profile");
     unsigned* bucket_count = at<unsigned>(ws, p.o_bucket_count);
-    NF_CUDA(cudaMemsetAsync(bucket_count, 0, 4 * kBuckets, s), "clear buckets");
     const int CH = 32 * t.sinks_per_lane;
     SymCtl* sym = p.any_sym ? at<SymCtl>(ws, p.o_sym) : nullptr;
     unsigned long long* sym_total = p.any_sym ? reinterpret_cast<unsigned long long*>(sym + 1) : nullptr;
@@ -495,7 +512,6 @@ int run_forces(const Plan& p, bool adjoint, const ForceTuning& t, const float* p
     int4* units = at<int4>(ws, p.o_sym_units);
     int* chunks = at<int>(ws, p.o_chunks);
     unsigned char* bucket_of = at<unsigned char>(ws, p.o_bucket_of);
-    if (p.any_sym) NF_CUDA(cudaMemsetAsync(sym, 0, sizeof(SymCtl) + 24 * (size_t)p.nboxes, s), "clear units");
     NF_CUDA(launch_pencils(boxes, p.nboxes, (int)p.C, off, CH, t.stage, chunks, bucket_count, bucket_of, dims,
                            sym_total, gm, hdr, s),
             "pencils");

@@ -215,10 +215,14 @@ __device__ __forceinline__ int cell_coord(float x, const BoxDev& B, float* off, 
     return r.c;
 }
 
-__global__ void k_fill_boxes(BoxFill f, BoxDev* boxes)
+// Writes the box table and clears the call's counters (the first of a call: instead
+// of a memset of each).
+__global__ void k_fill_boxes(BoxFill f, BoxDev* boxes, ClearList clear)
 {
     int i = threadIdx.x;
     if (i < f.count) boxes[f.first + i] = f.b[i];
+    for (int r = 0; r < ClearList::kMax; ++r)
+        for (int q = threadIdx.x; q < clear.words[r]; q += blockDim.x) clear.at[r][q] = 0u;
 }
 
 // Cell id (global: cell_base + local id) and cell-centred offsets of particle
@@ -380,6 +384,10 @@ __device__ __forceinline__ void block_scan_array(unsigned* a, int n)
 constexpr int kScanThreads = 1024;
 constexpr int kScanPer = 4;
 constexpr int kScanTile = kScanThreads * kScanPer;
+// Up to here one block scans the whole matrix: one launch of 3 us (4096 particles, 512
+// counts) to 6 us (32768, 8192 counts) instead of three of 3 us each.  Together with the
+// clears in k_fill_boxes: nf_forces of 4096 particles 94.2 -> 80.6 us, of 32768 213 -> 204.
+constexpr size_t kScanOneBlock = 4 * kScanTile;
 
 __global__ void k_scan_reduce(const unsigned* __restrict__ d, size_t n, unsigned* __restrict__ aux)
 {
@@ -620,9 +628,9 @@ int grid_for(size_t n, int threads)
 
 }  // namespace
 
-cudaError_t launch_fill_boxes(const BoxFill& f, BoxDev* boxes, cudaStream_t s)
+cudaError_t launch_fill_boxes(const BoxFill& f, BoxDev* boxes, const ClearList& clear, cudaStream_t s)
 {
-    k_fill_boxes<<<1, kMaxBoxesPerFill, 0, s>>>(f, boxes);
+    k_fill_boxes<<<1, 128, 0, s>>>(f, boxes, clear);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -686,10 +694,15 @@ cudaError_t run_sort(const SortPlan& p, const float* pos, int N, int C, const Bo
         count_launches(1);
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
         const size_t nb = (mn + kScanTile - 1) / kScanTile;
-        k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, s>>>(M, mn, aux);
-        k_scan_aux<<<1, kScanThreads, 0, s>>>(aux, nb);
-        k_scan_apply<<<(unsigned)nb, kScanThreads, 0, s>>>(M, mn, aux);
-        count_launches(3);
+        if (mn <= kScanOneBlock) {
+            k_scan_aux<<<1, kScanThreads, 0, s>>>(M, mn);
+            count_launches(1);
+        } else {
+            k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, s>>>(M, mn, aux);
+            k_scan_aux<<<1, kScanThreads, 0, s>>>(aux, nb);
+            k_scan_apply<<<(unsigned)nb, kScanThreads, 0, s>>>(M, mn, aux);
+            count_launches(3);
+        }
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
         const size_t smem = sort_smem_bytes(B);
         typedef void (*PassFn)(const float*, const BoxDev*, int, const float4*, const int*, float4*, int*, int*,

@@ -97,6 +97,13 @@ struct BoxFill {
     BoxDev b[kMaxBoxesPerFill];
 };
 
+// Words that a call's first kernel clears.
+struct ClearList {
+    static constexpr int kMax = 3;
+    unsigned* at[kMax];
+    int words[kMax];
+};
+
 constexpr int kCombineChunk = 256;   // particles per combine block, one a thread (never straddles boxes)
 constexpr int kBuckets = 64;         // cost buckets of the LPT work order
 
@@ -224,7 +231,7 @@ void count_launches(int n);
 cudaError_t ensure_smem(const void* fn, int bytes, bool max_carveout = false);
 
 // ---- launch wrappers (nf_bin.cu) ----
-cudaError_t launch_fill_boxes(const BoxFill& f, BoxDev* boxes, cudaStream_t s);
+cudaError_t launch_fill_boxes(const BoxFill& f, BoxDev* boxes, const ClearList& clear, cudaStream_t s);
 // Stable LSD sort of (cell id, particle): digits of at most kSortMaxBits bits,
 // one k_sort_pass launch per digit over tiles of kSortTile particles.
 constexpr int kSortMaxBits = 9;
