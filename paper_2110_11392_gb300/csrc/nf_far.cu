@@ -1072,19 +1072,10 @@ __global__ void k_far_rebuild(const void* __restrict__ Trv, int C, int p, int nt
         fd[i] = make_float4(x.h, x.l, y.h, y.l);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int i = 0;
-        for (int c = 0; c <= p; ++c) {
-            level[c] = i;
-            while (i < nt) {
-                int a, b, cz;
-                decode_term(prog[i].x, p, a, b, cz);
-                if (cz != c) break;
-                ++i;
-            }
-        }
-        level[p + 1] = nt;
-    }
+    // The program holds every term, by z index: those of z index >= c are the last
+    // far_terms(p - c).  (One thread that decoded the 165 terms in turn took most of a
+    // small grid's rebuild: 51.5 us at K = 11, p = 8, now 16.7.)
+    if ((int)threadIdx.x <= p + 1) level[threadIdx.x] = nt - far_terms(p - (int)threadIdx.x);
     __syncthreads();
     double t0 = 0.0;
     if (t002 >= 0 && partial)
@@ -1328,7 +1319,23 @@ struct ArDF {
 
 constexpr int kGPoints = 1024;  // complex points per buffer of one block
 
-__host__ __device__ inline int gfft_lines_per_block(int K) { return K >= kGPoints ? 1 : kGPoints / K; }
+// Lines per block: at most kGPoints points (enough work for 256 threads and two buffers
+// that leave six blocks per SM), fewer where a small grid would leave SMs without a block.
+// At K = 11 and 81 fields (5346 lines) a line pass takes 18 lines a block: 9.1 us, against
+// 32.3 us with the six lines of one (field, plane) to a block and a thread per line.
+inline int gfft_lines_per_block(int K, long long lines)
+{
+    const long long cap = K >= kGPoints ? 1 : kGPoints / K, want = (lines + 2 * device_sms() - 1) / (2 * device_sms());
+    return (int)(want < 1 ? 1 : want < cap ? want : cap);
+}
+
+// Fields per block of the z passes (one (x, y) column per block), by the same two rules.
+inline int gfft_fields_per_block(int K, int nf)
+{
+    const long long cap = K >= kGPoints ? 1 : kGPoints / K, cols = (long long)K * K;
+    const long long chunks = std::max((nf + cap - 1) / cap, (2 * device_sms() + cols - 1) / cols);
+    return (int)((nf + chunks - 1) / chunks);
+}
 
 template <class A, bool INV>
 __device__ __forceinline__ typename A::cx gtw(const typename A::cx* tw, int j)
@@ -1359,22 +1366,23 @@ __device__ __forceinline__ void gfft_step(const typename A::cx* a, typename A::c
     }
 }
 
-// The same for a radix known only at run time (a prime factor above 7).
+// Output m of the same step for a radix known only at run time (a prime factor above 7):
+// one thread per output, so that a line of prime length keeps R threads busy and not one.
 template <class A, bool INV>
-__device__ void gfft_step_any(const typename A::cx* a, typename A::cx* y, const typename A::cx* tw, int K, int R,
-                              int KR, int Ns, int j)
+__device__ void gfft_out_any(const typename A::cx* a, typename A::cx* y, const typename A::cx* tw, int R, int KR,
+                             int Ns, int j, int m)
 {
     typedef typename A::cx cx;
-    const int k = j % Ns, step = KR / Ns;
-    const int o = (j - k) * R + k;
-    for (int m = 0; m < R; ++m) {
-        cx acc = a[j];
-        for (int q = 1; q < R; ++q) {
-            const cx x = A::mul(gtw<A, INV>(tw, q * k * step), a[j + q * KR]);
-            acc = A::add(acc, A::mul(gtw<A, INV>(tw, ((q * m) % R) * KR), x));
-        }
-        y[o + m * Ns] = acc;
+    const int k = j % Ns, kstep = k * (KR / Ns);
+    cx acc = a[j];
+    int root = 0;
+    for (int q = 1; q < R; ++q) {
+        root += m;  // q m mod R
+        if (root >= R) root -= R;
+        const cx x = A::mul(gtw<A, INV>(tw, q * kstep), a[j + q * KR]);
+        acc = A::add(acc, A::mul(gtw<A, INV>(tw, root * KR), x));
     }
+    y[(j - k) * R + k + m * Ns] = acc;
 }
 
 // Transforms nl lines of K points in b0 (natural order); returns the buffer
@@ -1389,17 +1397,23 @@ __device__ typename A::cx* gfft_stages(typename A::cx* b0, typename A::cx* b1, i
     int Ns = 1;
     for (int st = 0; st < rd.n; ++st) {
         const int R = rd.r[st], KR = K / R;
-        for (int idx = threadIdx.x; idx < nl * KR; idx += blockDim.x) {
-            const int l = idx / KR, j = idx - l * KR;
-            const cx* a = src + (size_t)l * K;
-            cx* y = dst + (size_t)l * K;
-            switch (R) {
-                case 2: gfft_step<A, INV, 2>(a, y, tw, K, KR, Ns, j); break;
-                case 3: gfft_step<A, INV, 3>(a, y, tw, K, KR, Ns, j); break;
-                case 4: gfft_step<A, INV, 4>(a, y, tw, K, KR, Ns, j); break;
-                case 5: gfft_step<A, INV, 5>(a, y, tw, K, KR, Ns, j); break;
-                case 7: gfft_step<A, INV, 7>(a, y, tw, K, KR, Ns, j); break;
-                default: gfft_step_any<A, INV>(a, y, tw, K, R, KR, Ns, j); break;
+        if (R > 7) {
+            for (int idx = threadIdx.x; idx < nl * K; idx += blockDim.x) {
+                const int l = idx / K, jm = idx - l * K, j = jm / R;
+                gfft_out_any<A, INV>(src + (size_t)l * K, dst + (size_t)l * K, tw, R, KR, Ns, j, jm - j * R);
+            }
+        } else {
+            for (int idx = threadIdx.x; idx < nl * KR; idx += blockDim.x) {
+                const int l = idx / KR, j = idx - l * KR;
+                const cx* a = src + (size_t)l * K;
+                cx* y = dst + (size_t)l * K;
+                switch (R) {
+                    case 2: gfft_step<A, INV, 2>(a, y, tw, K, KR, Ns, j); break;
+                    case 3: gfft_step<A, INV, 3>(a, y, tw, K, KR, Ns, j); break;
+                    case 4: gfft_step<A, INV, 4>(a, y, tw, K, KR, Ns, j); break;
+                    case 5: gfft_step<A, INV, 5>(a, y, tw, K, KR, Ns, j); break;
+                    default: gfft_step<A, INV, 7>(a, y, tw, K, KR, Ns, j); break;
+                }
             }
         }
         __syncthreads();
@@ -1412,24 +1426,24 @@ __device__ typename A::cx* gfft_stages(typename A::cx* b0, typename A::cx* b1, i
 }
 
 // Shared memory of the generic kernels: the K twiddles, then two buffers of
-// (lines per block) x K points.
+// nl x K points, then the lines' first slots.
 template <class A>
-__host__ __device__ size_t gfft_smem(int K)
+size_t gfft_smem(int K, int nl)
 {
-    return sizeof(typename A::cx) * ((size_t)K + 2ull * gfft_lines_per_block(K) * K);
+    return sizeof(typename A::cx) * ((size_t)K + 2ull * nl * K) + 8ull * nl;
 }
 
 // Forward z pass: real fields R [x][y][z][nf] -> spectrum S [nf][x][y][kz].
 template <class A>
 __global__ void __launch_bounds__(kFftThreads) k_gfft_z_fwd(const typename A::real_t* __restrict__ Rf, int K, int nf,
-                                                            int nchunk, Radices rd,
+                                                            int FB, int nchunk, Radices rd,
                                                             const typename A::spec_t* __restrict__ twg,
                                                             typename A::spec_t* __restrict__ S)
 {
     typedef typename A::cx cx;
     extern __shared__ __align__(16) unsigned char gsm[];
     cx* tw = reinterpret_cast<cx*>(gsm);
-    const int FB = gfft_lines_per_block(K), H = K / 2 + 1;
+    const int H = K / 2 + 1;
     cx* b0 = tw + K;
     cx* b1 = b0 + (size_t)FB * K;
     const int chunk = blockIdx.x % nchunk;
@@ -1450,47 +1464,52 @@ __global__ void __launch_bounds__(kFftThreads) k_gfft_z_fwd(const typename A::re
     }
 }
 
-// Complex passes along y or x, in place on S (as k_fft_lines).
+// Complex passes along y or x, in place on S: the lines are numbered (field, a, kz), a
+// the other coordinate, and a block takes W consecutive ones.
 template <class A, bool INV>
 __global__ void __launch_bounds__(kFftThreads) k_gfft_lines(typename A::spec_t* __restrict__ S, int K, int nA,
-                                                            long long astride, long long pstride, int nchunk,
-                                                            Radices rd, const typename A::spec_t* __restrict__ twg)
+                                                            long long astride, long long pstride, long long lines,
+                                                            int W, Radices rd,
+                                                            const typename A::spec_t* __restrict__ twg)
 {
     typedef typename A::cx cx;
     extern __shared__ __align__(16) unsigned char gsm[];
     cx* tw = reinterpret_cast<cx*>(gsm);
-    const int W = gfft_lines_per_block(K), H = K / 2 + 1;
+    const int H = K / 2 + 1;
     cx* b0 = tw + K;
     cx* b1 = b0 + (size_t)W * K;
-    const int chunk = blockIdx.x % nchunk;
-    const long long fa = blockIdx.x / nchunk;
-    const long long f = fa / nA, a = fa - f * nA;
-    const int k0 = chunk * W, wc = min(W, H - k0);
+    long long* first = reinterpret_cast<long long*>(b1 + (size_t)W * K);
+    const long long l0 = (long long)blockIdx.x * W;
+    const int wc = (int)min((long long)W, lines - l0);
+    for (int w = threadIdx.x; w < wc; w += blockDim.x) {
+        const long long fa = (l0 + w) / H, f = fa / nA;
+        first[w] = f * (long long)K * K * H + (fa - f * nA) * astride + (l0 + w - fa * H);
+    }
     for (int j = threadIdx.x; j < K; j += blockDim.x) tw[j] = A::ld(twg[j]);
-    typename A::spec_t* base = S + f * (long long)K * K * H + a * astride + k0;
+    __syncthreads();
     for (int idx = threadIdx.x; idx < K * wc; idx += blockDim.x) {
         const int pt = idx / wc, w = idx - pt * wc;
-        b0[(size_t)w * K + pt] = A::ld(base[pt * pstride + w]);
+        b0[(size_t)w * K + pt] = A::ld(S[first[w] + pt * pstride]);
     }
     __syncthreads();
     const cx* out = gfft_stages<A, INV>(b0, b1, wc, K, rd, tw);
     for (int idx = threadIdx.x; idx < K * wc; idx += blockDim.x) {
         const int pt = idx / wc, w = idx - pt * wc;
-        base[pt * pstride + w] = A::st(out[(size_t)w * K + pt]);
+        S[first[w] + pt * pstride] = A::st(out[(size_t)w * K + pt]);
     }
 }
 
 // Inverse z pass: spectrum S (kz <= K/2) -> real fields R [x][y][z][nf].
 template <class A>
 __global__ void __launch_bounds__(kFftThreads) k_gfft_z_inv(const typename A::spec_t* __restrict__ S, int K, int nf,
-                                                            int nchunk, Radices rd,
+                                                            int FB, int nchunk, Radices rd,
                                                             const typename A::spec_t* __restrict__ twg,
                                                             typename A::real_t* __restrict__ Rf)
 {
     typedef typename A::cx cx;
     extern __shared__ __align__(16) unsigned char gsm[];
     cx* tw = reinterpret_cast<cx*>(gsm);
-    const int FB = gfft_lines_per_block(K), H = K / 2 + 1;
+    const int H = K / 2 + 1;
     cx* b0 = tw + K;
     cx* b1 = b0 + (size_t)FB * K;
     const int chunk = blockIdx.x % nchunk;
@@ -1526,30 +1545,31 @@ cudaError_t launch_gfft(int K, int nf, bool forward, const void* real_in, void* 
     typedef typename A::spec_t spec_t;
     typedef typename A::real_t real_t;
     const Radices rd = far_radices(K);
-    const int H = K / 2 + 1, FB = gfft_lines_per_block(K);
-    const size_t smem = gfft_smem<A>(K);
+    const int H = K / 2 + 1, FB = gfft_fields_per_block(K, nf);
+    const long long lines = (long long)nf * K * H, KH = (long long)K * H;
+    const int W = gfft_lines_per_block(K, lines);
+    const size_t zsmem = gfft_smem<A>(K, FB), lsmem = gfft_smem<A>(K, W);
     const spec_t* twg = static_cast<const spec_t*>(tw);
     spec_t* S = static_cast<spec_t*>(spec);
-    const int zchunks = (nf + FB - 1) / FB, lchunks = (H + FB - 1) / FB;
-    const long long zblocks = (long long)K * K * zchunks, lblocks = (long long)nf * K * lchunks;
-    const long long KH = (long long)K * H;
+    const int zchunks = (nf + FB - 1) / FB;
+    const unsigned zblocks = (unsigned)((long long)K * K * zchunks), lblocks = (unsigned)((lines + W - 1) / W);
     cudaError_t e;
     if (forward) {
-        e = ensure_smem((const void*)k_gfft_z_fwd<A>, (int)smem);
-        if (e == cudaSuccess) e = ensure_smem((const void*)k_gfft_lines<A, false>, (int)smem);
+        e = ensure_smem((const void*)k_gfft_z_fwd<A>, (int)zsmem);
+        if (e == cudaSuccess) e = ensure_smem((const void*)k_gfft_lines<A, false>, (int)lsmem);
         if (e != cudaSuccess) return e;
-        k_gfft_z_fwd<A><<<(unsigned)zblocks, kFftThreads, smem, s>>>(static_cast<const real_t*>(real_in), K, nf,
-                                                                      zchunks, rd, twg, S);
-        k_gfft_lines<A, false><<<(unsigned)lblocks, kFftThreads, smem, s>>>(S, K, K, KH, H, lchunks, rd, twg);
-        k_gfft_lines<A, false><<<(unsigned)lblocks, kFftThreads, smem, s>>>(S, K, K, H, KH, lchunks, rd, twg);
+        k_gfft_z_fwd<A><<<zblocks, kFftThreads, zsmem, s>>>(static_cast<const real_t*>(real_in), K, nf, FB, zchunks,
+                                                            rd, twg, S);
+        k_gfft_lines<A, false><<<lblocks, kFftThreads, lsmem, s>>>(S, K, K, KH, H, lines, W, rd, twg);
+        k_gfft_lines<A, false><<<lblocks, kFftThreads, lsmem, s>>>(S, K, K, H, KH, lines, W, rd, twg);
     } else {
-        e = ensure_smem((const void*)k_gfft_z_inv<A>, (int)smem);
-        if (e == cudaSuccess) e = ensure_smem((const void*)k_gfft_lines<A, true>, (int)smem);
+        e = ensure_smem((const void*)k_gfft_z_inv<A>, (int)zsmem);
+        if (e == cudaSuccess) e = ensure_smem((const void*)k_gfft_lines<A, true>, (int)lsmem);
         if (e != cudaSuccess) return e;
-        k_gfft_lines<A, true><<<(unsigned)lblocks, kFftThreads, smem, s>>>(S, K, K, H, KH, lchunks, rd, twg);
-        k_gfft_lines<A, true><<<(unsigned)lblocks, kFftThreads, smem, s>>>(S, K, K, KH, H, lchunks, rd, twg);
-        k_gfft_z_inv<A><<<(unsigned)zblocks, kFftThreads, smem, s>>>(S, K, nf, zchunks, rd, twg,
-                                                                      static_cast<real_t*>(real_out));
+        k_gfft_lines<A, true><<<lblocks, kFftThreads, lsmem, s>>>(S, K, K, H, KH, lines, W, rd, twg);
+        k_gfft_lines<A, true><<<lblocks, kFftThreads, lsmem, s>>>(S, K, K, KH, H, lines, W, rd, twg);
+        k_gfft_z_inv<A><<<zblocks, kFftThreads, zsmem, s>>>(S, K, nf, FB, zchunks, rd, twg,
+                                                            static_cast<real_t*>(real_out));
     }
     count_launches(3);
     return cudaGetLastError();
