@@ -355,7 +355,7 @@ def run_native(args, rank, world, local):
     traffic = kernel_traffic("force", args.workload)
     roofline = {"bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
                 "frac": achieved / fp32_peak, "traffic": traffic,
-                "kernel": "k_force (forward pair loop)",
+                "kernel": "forward pair loop (k_sym, which meets each unordered pair once, or k_force)",
                 "peak_basis": f"derived: {sms} SMs x 128 FP32 lanes x 2 flop x {max_mhz:.0f} MHz max SM clock",
                 "frac_at_sampled_clock": (achieved / (sms * 256 * clk["sm_mhz"] * 1e6 / 1e12)
                                           if clk.get("sm_mhz") else None),

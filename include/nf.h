@@ -193,10 +193,12 @@ typedef struct {
  *                   build at one block per SM).
  * Unsupported combinations are rejected with NF_ERR_ARG.  The built-in
  * defaults are below.  Under the built-in tuning of a direction, boxes of 2^18
- * to 2^28 particles run in the symmetric kernel, which meets every pair once and
- * applies it to both particles, unless much of a box's work lies in a few dense
- * pencils (decided on the device, per box); any other tuning, and the time
- * steps, run the directed kernel that it shapes. */
+ * to 2^28 particles (above the sizes of nf_forces_noalloc) run in the symmetric
+ * kernel, which meets every pair once and applies it to both particles, where
+ * their pencils hold enough sinks to fill its lanes and no few dense pencils hold
+ * much of the work (decided on the device, per box).  The others, any other
+ * tuning and the time steps run the directed kernel that the tuning shapes; on a
+ * small box the warps of one of its blocks share an item. */
 typedef struct {
     int sinks_per_lane;
     int stage;

@@ -15,7 +15,7 @@
 // of cells once.  The centre cell meets the sinks with c < 0 (both get the
 // force) and itself (c = 0: ordered pairs, one-sided).  A particle collects
 // 2R+1 partial sums as a sink and 1 + ((2R+1)^2 - 1)/2 as a source, each in a
-// slot of its own; k_combine_sym adds them without rounding error.  No result
+// slot of its own; k_combine adds them without rounding error.  No result
 // depends on the order in which warps run.
 //
 // One warp runs one unit: the pencil's sinks (in chunks of 64 G, two per lane
@@ -33,9 +33,9 @@
 // rule on N, with slots of their own for the sinks); where even a run is dearer
 // than one warp's share of the box, the sinks' half and the sources' half of
 // the work become one-sided units per chunk (22 operations a pair instead of
-// 14, any number of warps).  A box with much of its work in such pencils is left
-// to the directed kernel (box_is_sym, on the device: the counts are not known on
-// the host).
+// 14, any number of warps).  A box with much of its work in such pencils, or whose
+// pencils fill the lanes badly, is left to the directed kernel (box_is_sym, on the
+// device: the counts are not known on the host).
 //
 // Softening and the density follow nf_force.cu: tiles that can hold a pair
 // closer than a cell track the smallest r^2 and are run again on the exact
