@@ -20,7 +20,7 @@ SOURCES = ["nf_bin.cu", "nf_force.cu", "nf_sym.cu", "nf_step.cu", "nf_multipole.
 # the benchmark's multiply-add probe: a library of its own, not part of libnf
 PROBE_SRC = os.path.join(CSRC, "probe", "fma_probe.cu")
 PROBE_LIB = os.path.join(PKG, "libnf_probe.so")
-HEADERS = ["nf_internal.cuh", "nf_pair.cuh"]
+HEADERS = ["nf_internal.cuh", "nf_pair.cuh", "nf_cell.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 LINK_LIBS: List[str] = []
 NVCC_FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]

@@ -32,6 +32,7 @@
 #include <algorithm>
 #include <cstdio>
 
+#include "nf_cell.cuh"
 #include "nf_internal.cuh"
 
 namespace nf {
@@ -181,33 +182,8 @@ __device__ __forceinline__ int cell_coord(float x, const BoxDev& B, float* off, 
             return ci % B.K;
         }
     } else {
-        // Any other K / box: t = x K/box as a float pair p + e, within err of the FP64
-        // product (kl_hi + kl_lo is K / box to 2^-48).  p - c is exact and, unless p is an
-        // integer, inside (0, 1) by more than |e|, so c = floor(t).  The offset is the sum
-        // rounded to 24 bits, taken where no value within err rounds otherwise; the few
-        // others (near a rounding boundary, a face or a cell centre) take the integer path.
-        // A third of that path's instructions.
-        const float p = __fmul_rn(x, B.kl_hi);
-        if (p >= 0.000244140625f && p < 1048576.0f) {  // false for NaN and when kl_hi is 0
-            const float c = floorf(p), f = __fsub_rn(p, c);
-            const int ci = (int)c;
-            if constexpr (!OFF) {
-                if (f > 0.0f) return ci < B.K ? ci : ci % B.K;
-            } else {
-                const float e = __fmaf_rn(x, B.kl_lo, __fmaf_rn(x, B.kl_hi, -p));
-                const float a = __fsub_rn(f, 0.5f);
-                // f - 1/2 - a, exact: |f| <= 1/2 wherever a is rounded
-                const float tail = __fadd_rn(__fsub_rn(f, __fadd_rn(a, 0.5f)), e);
-                const float o = __fadd_rn(a, tail);
-                const float r = __fsub_rn(tail, __fsub_rn(o, a));
-                const float err = __fmaf_rn(p, 1.4210854715202004e-14f, 8.8817841970012523e-16f);  // 2^-46 p + 2^-50
-                if (f > 0.0f && fabsf(a) >= 0.000244140625f && __fadd_rn(o, __fadd_rn(r, err)) == o &&
-                    __fadd_rn(o, __fsub_rn(r, err)) == o) {
-                    *off = o;
-                    return ci < B.K ? ci : ci % B.K;
-                }
-            }
-        }
+        int ci;
+        if (cell_short<OFF>(x, B.kl_hi, B.kl_lo, &ci, off)) return ci < B.K ? ci : ci % B.K;
     }
     const CellCoord r = cell_coord_general<OFF>(x, B.K, B.kl_mant, B.kl_exp, B.kl);
     if constexpr (OFF) *off = r.off;
