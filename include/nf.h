@@ -77,7 +77,12 @@ const char *nf_version(void);
 /* Bytes of device workspace that nf_bin, nf_forces and nf_forces_adjoint need
  * for one box of N particles on a K^3 grid with radius R.  Returns 0 for
  * arguments nf_forces would reject.  The workspace's first 256 bytes hold the
- * device status word read by nf_status_read. */
+ * device status word read by nf_status_read.
+ * Bytes per particle at R = 2 and 64 particles per cell: 141 where only the
+ * directed kernel can run; where the symmetric one may (nf_tuning), whose partial
+ * sums have 18 to 53 slots a particle, 929 up to 1.5 10^6 particles, 602 at 128^3,
+ * 440 at 256^3 and 357 at 512^3 (R = 4: 2104 down to 209, the directed kernel's,
+ * above 10^8). */
 size_t nf_workspace_bytes(int64_t N, int K, int R);
 
 /* ------------------------------------------------------------------------ */
@@ -193,7 +198,8 @@ typedef struct {
  *                   build at one block per SM).
  * Unsupported combinations are rejected with NF_ERR_ARG.  The built-in
  * defaults are below.  Under the built-in tuning of a direction, boxes of 2^18
- * to 2^28 particles (above the sizes of nf_forces_noalloc) run in the symmetric
+ * to 2^28 particles (above the sizes of nf_forces_noalloc, and with partial sums of
+ * 80 GB at most, which excludes more than 10^8 at R = 4) run in the symmetric
  * kernel, which meets every pair once and applies it to both particles, where
  * their pencils hold enough sinks to fill its lanes and no few dense pencils hold
  * much of the work (decided on the device, per box).  The others, any other
@@ -220,7 +226,10 @@ void nf_get_default_tuning(nf_tuning *t);
 int nf_set_default_tuning_adjoint(const nf_tuning *t);
 void nf_get_default_tuning_adjoint(nf_tuning *t);
 
-/* Workspace for a batch (host array boxes[nboxes]); 0 if the batch is invalid. */
+/* Workspace for a batch (host array boxes[nboxes]); 0 if the batch is invalid.
+ * The boxes share the symmetric kernel's partial sums: 8 GiB of them at most, or
+ * what the largest box needs alone, beside the directed kernel's.  Boxes that do
+ * not fit side by side run in rounds. */
 size_t nf_workspace_bytes_batched(const nf_box *boxes, int nboxes);
 
 /* Near-field accelerations of nboxes independent periodic boxes in one pass:

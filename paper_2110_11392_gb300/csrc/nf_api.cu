@@ -164,20 +164,28 @@ size_t directed_bytes(int64_t N, int64_t C, int R)
 // whose fixed scratch cannot hold the partial planes and whose results are
 // nf_forces'.  From 64^3 particles on it is the faster one (pair kernel, clustered:
 // forward 0.89 against 0.99 ms, adjoint 1.59 against 1.80); a smaller box has too few
-// pencils for its warps.  Above, the planes (18 slots of 16 bytes a particle at R = 2)
-// would take over 80 GB.  The time steps stay on the directed kernel: the step size
+// pencils for its warps.  Above, or where a wide stencil has many slots, the planes (18
+// slots of 16 bytes a particle at R = 2, 50 at R = 4) would take over 80 GB.  The time steps stay on the directed kernel: the step size
 // they write is a double made of a few of the FP32 accelerations, read back by the
 // next step, so the last bits of the sums decide a run's trajectory, and a run
 // continued with this version keeps it.
 constexpr int64_t kSymMinN = int64_t(1) << 18, kSymMaxN = int64_t(1) << 28;
+constexpr int64_t kSymMaxPlaneBytes = 80000000000;
+// The boxes of a batch share planes of this size (or of its largest box): those that do
+// not fit side by side run in rounds, one after the other on the same planes, so that a
+// batch of many boxes needs little more than its directed rows (300 boxes of 10^6
+// particles: 51 GB; 300 GB with planes for all).
+constexpr int64_t kSymRoundPlaneBytes = int64_t(8) << 30;
 // A box whose pencils hold too few sinks at mean occupancy for the symmetric
 // kernel's lanes (fill_needed) is not considered: the choice costs two launches.
+int sym_box_groups(int64_t N);
+int64_t sym_plane_bytes(int64_t N, int R) { return 16 * (int64_t)sym_slots(R, sym_box_groups(N)) * N; }
 bool sym_box(const nf_box& b, bool adjoint)
 {
     const int64_t cells = (int64_t)b.K * b.K * b.K;
     const double sinks = (2.0 * b.R + 1.0) * (double)b.N / (double)cells;
     const double needed = b.N >= 1500000 ? 160.0 : adjoint ? 180.0 : b.N >= 450000 ? 260.0 : 430.0;
-    return b.N >= kSymMinN && b.N <= kSymMaxN && sinks >= needed &&
+    return b.N >= kSymMinN && b.N <= kSymMaxN && sinks >= needed && sym_plane_bytes(b.N, b.R) <= kSymMaxPlaneBytes &&
            directed_bytes(b.N, cells, b.R) > (size_t)NF_NOALLOC_SCRATCH_BYTES;
 }
 // Which boxes a plan may give to the symmetric kernel.
@@ -228,6 +236,11 @@ struct Plan {
     int max_nseg = 9;
     int nchunks = 0;     // combine chunks
     bool any_sym = false;  // boxes that may run in the symmetric pair kernel
+    // rounds of the symmetric boxes: consecutive boxes, by their cells and combine chunks
+    struct Round {
+        int c0, c1, chunk0, chunk1;
+    };
+    std::vector<Round> rounds;
     SortPlan sp{};
     std::vector<BoxDev> boxes;
     // region offsets (bytes from ws)
@@ -295,7 +308,7 @@ int make_plan(const nf_box* boxes, int nboxes, bool need_force, int chunk_lanes,
     if (!boxes || nboxes < 1) return fail(NF_ERR_ARG, "need at least one box");
     p->nboxes = nboxes;
     p->boxes.resize(nboxes);
-    int64_t N = 0, C = 0, items = 0, nchunks = 0, units = 0, planes = 0;
+    int64_t N = 0, C = 0, items = 0, nchunks = 0, units = 0, partials = 0;
     p->any_sym = false;
     p->mean_items = p->mean_stages = 0;
     int max_R = 1;
@@ -321,7 +334,6 @@ int make_plan(const nf_box* boxes, int nboxes, bool need_force, int chunk_lanes,
             if (sym != Sym::no && sym_box(boxes[b], sym == Sym::adjoint)) {
                 d.sym = 1;
                 d.groups = sym_box_groups(d.N);
-                units += sym_max_units(d.N, cells, d.R, d.groups);
                 p->any_sym = true;
             }
             items += directed_items(d.N, cells, d.R, chunk_lanes);
@@ -333,7 +345,7 @@ int make_plan(const nf_box* boxes, int nboxes, bool need_force, int chunk_lanes,
         if (N >= (int64_t(1) << 31)) return fail(NF_ERR_ARG, "total N must be < 2^31");
         if (C >= (int64_t(1) << 31) - 1) return fail(NF_ERR_ARG, "total cells must be < 2^31");
     }
-    if (items >= (int64_t(1) << 31) || units >= (int64_t(1) << 31)) return fail(NF_ERR_ARG, "too many work items");
+    if (items >= (int64_t(1) << 31)) return fail(NF_ERR_ARG, "too many work items");
     p->N = N;
     p->C = C;
     p->max_items = items;
@@ -341,15 +353,31 @@ int make_plan(const nf_box* boxes, int nboxes, bool need_force, int chunk_lanes,
     p->max_nseg = (2 * max_R + 1) * (2 * max_R + 1);
     p->nchunks = (int)nchunks;
     if (need_force) {
-        // partial sums: every particle's row (directed), then the planes of the symmetric boxes;
-        // a single box uses one or the other, so both start at the same place
-        const int64_t rows = 4 * (2 * (int64_t)max_R + 1) * N;
-        planes = rows;
+        // partial sums in bytes: every particle's row (directed), then the planes of a round's
+        // symmetric boxes; a single box uses one or the other, so both start at the same place
+        partials = 16 * (2 * (int64_t)max_R + 1) * N;
+        const int64_t first = nboxes == 1 ? 0 : partials;
+        int64_t planes = 0, round_units = 0;
+        p->rounds.assign(1, Plan::Round{0, 0, 0, 0});
         for (BoxDev& d : p->boxes) {
-            if (!d.sym) continue;
-            const int64_t size = 4 * (int64_t)sym_slots(d.R, d.groups) * d.N;
-            d.plane_base = nboxes == 1 ? 0 : planes;
-            planes = std::max<int64_t>(planes, d.plane_base + size);
+            Plan::Round* r = &p->rounds.back();
+            const int cells = d.K * d.K * d.K;
+            if (d.sym) {
+                const int64_t size = sym_plane_bytes(d.N, d.R);
+                if (planes > 0 && planes + size > kSymRoundPlaneBytes) {
+                    p->rounds.push_back(Plan::Round{r->c1, r->c1, r->chunk1, r->chunk1});
+                    r = &p->rounds.back();
+                    planes = round_units = 0;
+                }
+                d.round = (int)p->rounds.size() - 1;
+                d.plane_base = (first + planes) / 4;
+                planes += size;
+                round_units += sym_max_units(d.N, cells, d.R, d.groups);
+                partials = std::max(partials, first + planes);
+                units = std::max(units, round_units);
+            }
+            r->c1 = d.cell_base + cells;
+            r->chunk1 = d.chunk_base + (d.N + kCombineChunk - 1) / kCombineChunk;
         }
     }
     p->sp = sort_plan(N, C);
@@ -381,7 +409,7 @@ int make_plan(const nf_box* boxes, int nboxes, bool need_force, int chunk_lanes,
         p->o_bucket_count = take(4 * kBuckets);
         p->o_items = take(16 * (size_t)items);
         p->o_gs = take(16 * (size_t)N);
-        p->o_partial = take(4 * (size_t)planes);
+        p->o_partial = take((size_t)partials);
         p->o_sym = p->any_sym ? take(sizeof(SymCtl) + 24 * (size_t)nboxes) : 0;
         p->o_sym_dims = p->any_sym ? take(8 * (size_t)C) : 0;
         p->o_sym_units = p->any_sym ? take(16 * (size_t)units) : 0;
@@ -516,10 +544,14 @@ int run_forces(const Plan& p, bool adjoint, const ForceTuning& t, const float* p
                            sym_total, gm, hdr, s),
             "pencils");
     int4* items = at<int4>(ws, p.o_items);
+    // the symmetric boxes' work list, round by round (the directed list with the first)
+    auto sym_units = [&](int round) {
+        const Plan::Round& r = p.rounds[round];
+        return launch_sym_units(adjoint, boxes, p.nboxes, round, r.c0, round == 0 ? (int)p.C : r.c1, off, dims, sym,
+                                sym_total, units, chunks, bucket_of, bucket_count, items, hdr, s);
+    };
     if (p.any_sym) {
-        NF_CUDA(launch_sym_units(adjoint, boxes, p.nboxes, (int)p.C, off, dims, sym, sym_total, units, chunks,
-                                 bucket_of, bucket_count, items, hdr, s),
-                "work units");
+        NF_CUDA(sym_units(0), "work units");
     } else {
         NF_CUDA(launch_bucket_scan(bucket_count, hdr, s), "work items");
         NF_CUDA(launch_items(boxes, p.nboxes, (int)p.C, chunks, bucket_of, bucket_count, items, hdr, s),
@@ -530,19 +562,30 @@ int run_forces(const Plan& p, bool adjoint, const ForceTuning& t, const float* p
     float4* partial = at<float4>(ws, p.o_partial);
     const int pstride = 2 * p.max_R + 1;  // partial row of a particle: one float4 per pencil slot
     NF_CUDA(prof_mark(2, s), "profile");
-    if (p.any_sym)
-        NF_CUDA(launch_sym_force(adjoint, rho != nullptr, boxes, off, rel, gs, units, sym, hdr,
-                                 reinterpret_cast<float*>(partial), s),
-                adjoint ? "symmetric adjoint kernel" : "symmetric force kernel");
+    auto sym_force = [&]() {
+        return launch_sym_force(adjoint, rho != nullptr, boxes, off, rel, gs, units, sym, hdr,
+                                reinterpret_cast<float*>(partial), s);
+    };
+    const char* sym_name = adjoint ? "symmetric adjoint kernel" : "symmetric force kernel";
+    if (p.any_sym) NF_CUDA(sym_force(), sym_name);
     // (with nothing on its list where every box is symmetric)
     const int coop = builtin_tuning(t, adjoint) && !p.any_sym ? coop_warps(p.mean_items, p.mean_stages, adjoint) : 1;
     NF_CUDA(launch_force(adjoint, rho != nullptr, t, coop, boxes, off, rel, gs, items, hdr, partial,
                          pstride, p.max_nseg, s),
             adjoint ? "adjoint kernel" : "force kernel");
-    NF_CUDA(prof_mark(3, s), "profile");
     double* chunk_sums = net ? at<double>(ws, p.o_chunk_sums) : nullptr;
-    NF_CUDA(launch_combine(adjoint, boxes, p.nboxes, p.nchunks, partial, pstride, perm, out, rho, chunk_sums, s),
-            "combine");
+    auto combine = [&](const Plan::Round& r) {
+        return launch_combine(adjoint, boxes, p.nboxes, r.chunk0, r.chunk1 - r.chunk0, partial, pstride, perm, out,
+                              rho, chunk_sums, s);
+    };
+    // each round's planes are combined before the next one writes them
+    for (size_t q = 1; q < p.rounds.size(); ++q) {
+        NF_CUDA(combine(p.rounds[q - 1]), "combine");
+        NF_CUDA(sym_units((int)q), "work units");
+        NF_CUDA(sym_force(), sym_name);
+    }
+    NF_CUDA(prof_mark(3, s), "profile");
+    NF_CUDA(combine(p.rounds.back()), "combine");
     if (net) NF_CUDA(launch_net(boxes, p.nboxes, chunk_sums, net, s), "net force");
     NF_CUDA(prof_mark(4, s), "profile");
     if (g_profile_on) ++g_prof_count;

@@ -929,13 +929,13 @@ k_force(const BoxDev* __restrict__ boxes, const int* __restrict__ off, const flo
 // (16 rounds in a row on a few blocks); with one round the whole nf_forces
 // call of 4096 particles went from 171 to 158 us, of 32768 from 279 to 264.
 __global__ void __launch_bounds__(kCombineChunk)
-k_combine(const BoxDev* __restrict__ boxes, int nboxes, const float4* __restrict__ partial, int pstride,
+k_combine(const BoxDev* __restrict__ boxes, int nboxes, int chunk0, const float4* __restrict__ partial, int pstride,
           const int* __restrict__ perm, float* __restrict__ out, float* __restrict__ rho,
           double* __restrict__ chunk_sums, bool adjoint)
 {
     // block = one chunk of particles of a single box
     __shared__ double red[3][kCombineChunk / 32];
-    int chunk = blockIdx.x;
+    int chunk = chunk0 + blockIdx.x;
     int lo = 0, hi = nboxes - 1;
     while (lo < hi) {
         int mid = (lo + hi + 1) >> 1;
@@ -1226,11 +1226,13 @@ cudaError_t launch_force(bool adjoint, bool density, const ForceTuning& t, int c
     return cudaGetLastError();
 }
 
-cudaError_t launch_combine(bool adjoint, const BoxDev* boxes, int nboxes, int nchunks, const float4* partial,
-                           int pstride, const int* perm, float* out, float* rho, double* chunk_sums, cudaStream_t s)
+cudaError_t launch_combine(bool adjoint, const BoxDev* boxes, int nboxes, int chunk0, int nchunks,
+                           const float4* partial, int pstride, const int* perm, float* out, float* rho,
+                           double* chunk_sums, cudaStream_t s)
 {
     if (nchunks <= 0) return cudaSuccess;
-    k_combine<<<nchunks, kCombineChunk, 0, s>>>(boxes, nboxes, partial, pstride, perm, out, rho, chunk_sums, adjoint);
+    k_combine<<<nchunks, kCombineChunk, 0, s>>>(boxes, nboxes, chunk0, partial, pstride, perm, out, rho, chunk_sums,
+                                                adjoint);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -56,7 +56,9 @@ struct BoxDev {
     float kl_pow2;
     // K / box as a float pair, or 0 outside FP32's middle range
     float kl_hi, kl_lo;
-    int pad[2];
+    // pass over the batch in which a symmetric box runs (make_plan)
+    int round;
+    int pad;
     // 1: the top-hat term runs only in the pair-kernel stages where some pair
     // is closer than b (small b); 0: it is fused into every stage that can hold one
     int dens_defer;
@@ -283,8 +285,9 @@ cudaError_t launch_force(bool adjoint, bool density, const ForceTuning& t, int c
                          const int4* items, WsHeader* hdr, float4* partial, int pstride,
                          int max_nseg, cudaStream_t s);
 // partial: rows of pstride float4 (2 max R + 1) per particle in original order (directed
-// boxes), or planes per slot and component in sorted order (symmetric ones)
-cudaError_t launch_combine(bool adjoint, const BoxDev* boxes, int nboxes, int nchunks,
+// boxes), or planes per slot and component in sorted order (symmetric ones); combine
+// chunks [chunk0, chunk0 + nchunks)
+cudaError_t launch_combine(bool adjoint, const BoxDev* boxes, int nboxes, int chunk0, int nchunks,
                            const float4* partial, int pstride, const int* perm, float* out,
                            float* rho, double* chunk_sums, cudaStream_t s);
 cudaError_t launch_net(const BoxDev* boxes, int nboxes, const double* chunk_sums,
@@ -299,8 +302,10 @@ long long sym_max_units(long long N, long long C, int R, int groups);
 // total: [3 nboxes], the boxes' costs, the costs of their dear pencils (written here), and
 // the directed kernel's lane pairs.
 // Clears .sym of the boxes that run better directed; writes both lists (bucket_count holds
-// the other boxes' chunks).
-cudaError_t launch_sym_units(bool adjoint, BoxDev* boxes, int nboxes, int Ctot, const int* cell_off,
+// the other boxes' chunks).  Round 0 takes all cells [0, c1) and writes the directed list
+// whole; a later one, its boxes' cells [c0, c1).  units and ctl (cleared here after round
+// 0) hold one round's list.
+cudaError_t launch_sym_units(bool adjoint, BoxDev* boxes, int nboxes, int round, int c0, int c1, const int* cell_off,
                              const int2* dims, SymCtl* ctl, unsigned long long* total, int4* units,
                              const int* chunks, const unsigned char* bucket_of, unsigned* bucket_count, int4* items,
                              WsHeader* hdr, cudaStream_t s);
