@@ -85,6 +85,11 @@ const char *nf_version(void);
  * above 10^8). */
 size_t nf_workspace_bytes(int64_t N, int K, int R);
 
+/* Bytes that the calls which only sort need: nf_bin, nf_multipoles and
+ * nf_timestep (about 44 per particle and 4 per cell; they take any larger
+ * workspace too).  Returns 0 for arguments nf_bin would reject. */
+size_t nf_bin_workspace_bytes(int64_t N, int K);
+
 /* ------------------------------------------------------------------------ */
 /* Binning (Sec. "Force Accuracy" overview: FP32 offsets from cell centres;  */
 /* Sec. "Two-Stage Execution": the K^3 cell grid)                            */

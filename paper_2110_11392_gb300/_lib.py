@@ -77,6 +77,7 @@ def load(build: bool = True) -> ctypes.CDLL:
         "nf_last_error": (ctypes.c_char_p, []),
         "nf_version": (ctypes.c_char_p, []),
         "nf_workspace_bytes": (sz, [i64, i32, i32]),
+        "nf_bin_workspace_bytes": (sz, [i64, i32]),
         "nf_workspace_bytes_batched": (sz, [P, i32]),
         "nf_bin": (i32, [P, i64, f64, i32, P, P, P, P, sz, P]),
         "nf_forces": (i32, [P, i64, f64, i32, i32, f64, P, P, P, sz, P]),
@@ -122,7 +123,8 @@ def load(build: bool = True) -> ctypes.CDLL:
 
 
 def exported_symbols() -> Sequence[str]:
-    return ("nf_last_error", "nf_version", "nf_workspace_bytes", "nf_workspace_bytes_batched",
+    return ("nf_last_error", "nf_version", "nf_workspace_bytes", "nf_bin_workspace_bytes",
+            "nf_workspace_bytes_batched",
             "nf_bin", "nf_forces", "nf_forces_adjoint", "nf_forces_batched",
             "nf_forces_adjoint_batched", "nf_set_default_tuning", "nf_get_default_tuning",
             "nf_set_default_tuning_adjoint", "nf_get_default_tuning_adjoint",
@@ -175,6 +177,10 @@ def make_boxes(boxes) -> "ctypes.Array":
         arr[i].R = int(b.get("R", 2))
         off += int(b["N"])
     return arr
+
+
+def nf_bin_workspace_bytes(N: int, K: int) -> int:
+    return int(load().nf_bin_workspace_bytes(int(N), int(K)))
 
 
 def nf_workspace_bytes_batched(boxes) -> int:

@@ -716,6 +716,13 @@ size_t nf_workspace_bytes(int64_t N, int K, int R)
     return force_workspace_bytes(&b, 1);
 }
 
+size_t nf_bin_workspace_bytes(int64_t N, int K)
+{
+    nf_box b = one_box(N, 1.0, K, 0, 0.0);
+    Plan p;
+    return make_plan(&b, 1, false, 32, &p) ? 0 : p.total;
+}
+
 size_t nf_workspace_bytes_batched(const nf_box* boxes, int nboxes)
 {
     return force_workspace_bytes(boxes, nboxes);

@@ -47,7 +47,7 @@ def bin_particles(pos: torch.Tensor, box: float, K: int, ws: Optional[torch.Tens
     rel = torch.empty((N, 4), dtype=torch.float32, device=dev)
     perm = torch.empty(N, dtype=torch.int32, device=dev)
     if ws is None:
-        ws = workspace(_lib.nf_workspace_bytes(N, max(K, 5), 2), dev)
+        ws = workspace(_lib.nf_bin_workspace_bytes(N, K), dev)
     _lib.nf_bin(pos, box, K, off, rel, perm, ws)
     return off, rel, perm
 
@@ -104,7 +104,7 @@ def multipoles(pos: torch.Tensor, box: float, K: int, p: int, ws: Optional[torch
     pos = _check_pos(pos)
     N = pos.shape[0]
     if ws is None:
-        ws = workspace(_lib.nf_workspace_bytes(N, max(K, 5), 2), pos.device)
+        ws = workspace(_lib.nf_bin_workspace_bytes(N, K), pos.device)
     M = torch.empty((K ** 3, (p + 3) * (p + 2) * (p + 1) // 6), dtype=torch.float64, device=pos.device)
     _lib.nf_multipoles(pos, box, K, p, M, ws)
     return M

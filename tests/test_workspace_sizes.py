@@ -33,3 +33,27 @@ def test_one_box(N, K, R):
     need = _lib.nf_workspace_bytes(N, K, R)
     # the planes of a box are within 80 GB and may take the place of its rows
     assert 0 < need <= 1.05 * directed_bytes(N, K, R) + 84e9, need
+
+
+def test_sorting_alone_needs_no_partial_sums():
+    # keys 8, offsets between passes 16, offsets 16, permutation 4, and the sort's counts (one word per digit value
+    # and tile of 2048 particles, 9-bit digits at most): 45 bytes a particle; the cells' offsets
+    for N, K in ((60000000, 100), (20000000, 64), (1000, 4)):
+        need = _lib.nf_bin_workspace_bytes(N, K)
+        assert 0 < need <= 45.5 * N + 4 * K ** 3 + 65536, (N, K, need)
+    assert _lib.nf_bin_workspace_bytes(0, 8) == 0 and _lib.nf_bin_workspace_bytes(1000, 1291) == 0
+
+
+@pytest.mark.gpu
+def test_binning_keeps_a_workspace_of_its_own_size():
+    import torch
+    import paper_2110_11392_gb300 as nf
+    from paper_2110_11392_gb300 import nearfield
+    nearfield._WS_CACHE.clear()
+    N, K = 1 << 20, 25
+    pos = torch.rand((N, 3), device="cuda")
+    nf.bin_particles(pos, 1.0, K)
+    nf.multipoles(pos, 1.0, K, 2)
+    assert nf.workspace(0).numel() == _lib.nf_bin_workspace_bytes(N, K)
+    nf.forces(pos, 1.0, K, 2, 1e-4)  # grows it
+    assert nf.workspace(0).numel() == _lib.nf_workspace_bytes(N, K, 2)
