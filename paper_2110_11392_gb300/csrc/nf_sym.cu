@@ -64,6 +64,16 @@ namespace {
 constexpr int kGroupsFwd = 3, kBlocksFwd = 2;
 constexpr int kGroupsAdj = 5, kBlocksAdj = 1;
 constexpr int kWarps = 8;
+// Chains in which a resident's tile sums are added, tile t in chain t mod kChains (a power
+// of two).  One chain over all tiles of a pencil (26 at 64 particles per cell, hundreds in a
+// dense pencil) lost up to 8 % against the directed kernel in the median error; four
+// have a sixteenth of its variance and stay below the directed kernel.  Median error of
+// symmetric over directed with one, two and four chains: forward 2 10^6 uniform 1.06, 0.86,
+// 0.81, 36 10^6 clustered 1.07, 0.86, 0.79; adjoint 1.4 10^6 uniform 1.07, 0.98, 0.95,
+// 17 10^6 clustered 1.07, 0.97, 0.92, R = 3 1.08, 0.95, 0.88.  Call times with four over
+// one: forward 1.003, adjoint 256^3 1.008, 64^3 1.03.  Folding every eight tiles into a
+// second sum has the same errors and takes as long or longer.
+constexpr int kChains = 4;
 
 // (the density build cuts its chunks as the plain one does: its accelerations are the same bits)
 constexpr int sym_groups_max(bool adj) { return adj ? kGroupsAdj : kGroupsFwd; }
@@ -537,10 +547,10 @@ __device__ __forceinline__ void tile_adj_exact(const Tile& v, Residents<G, true>
 }
 
 // Per-warp shared memory: the tile (and its g), the cp.async targets, the
-// residents' running sums and the segment tables of both lists.
+// residents' running sums (kChains of them, and the density's) and the segment tables of
+// both lists.
 template <int GM, bool ADJ, bool DENS>
 struct SymSmem {
-    static constexpr int NS = DENS ? 4 : 3;
     static constexpr size_t xy = 0;
     static constexpr size_t z = xy + 64 * 16;
     static constexpr size_t gxy = z + 64 * 8;
@@ -548,7 +558,9 @@ struct SymSmem {
     static constexpr size_t raw = gz + (ADJ ? 64 * 8 : 0);
     static constexpr size_t graw = raw + 32 * 16;
     static constexpr size_t tot = graw + (ADJ ? 32 * 16 : 0);
-    static constexpr size_t tab = tot + (size_t)GM * NS * 32 * 8;
+    static constexpr int chain = GM * 3 * 32;  // sums of one chain
+    static constexpr size_t totw = tot + (size_t)kChains * chain * 8;
+    static constexpr size_t tab = totw + (DENS ? (size_t)GM * 32 * 8 : 0);
     static constexpr int NA = 2 * NF_MAX_R + 1;
     static constexpr size_t ints = (NA + 1) + NA + (kHalfMax + 1) + 2 * kHalfMax;
     static constexpr size_t bytes = (tab + 4 * ints + 15) & ~size_t(15);
@@ -660,8 +672,8 @@ __device__ __forceinline__ void run_pass(const Pass& ps, int R, const Coef& cf, 
     const bool soft_near_only = cf.eps2 <= 1.0f;  // eps_s <= one cell width
     const bool dens_defer = DENS && cf.dens_defer != 0 && dens_near_only;
     const Tile tv = {xy + lane, zz + lane, gxy + lane, gz + lane};
-    constexpr int TS = L::NS * 32;
-    f2* totw = tot + (DENS ? 96 : 0);
+    constexpr int TS = 32;
+    f2* totw = reinterpret_cast<f2*>(sm + L::totw) + lane;
     if constexpr (DENS)
 #pragma unroll
         for (int s = 0; s < G; ++s) totw[s * TS] = 0ull;
@@ -747,11 +759,12 @@ __device__ __forceinline__ void run_pass(const Pass& ps, int R, const Coef& cf, 
                 if (!dens || fused) tile_fwd_exact<G, REACT, false, TS>(tv, k, a, cf, b2, ms, mr, n_self, totw);
             }
         }
-        // the tile's sums join the running ones (chains of at most 32 sources)
+        // the tile's sums (chains of at most 32 sources) join one of the running ones
+        f2* const chain = tot + (t & (kChains - 1)) * L::chain;
 #pragma unroll
         for (int s = 0; s < G; ++s) {
-            f2* p = tot + (size_t)s * L::NS * 32;
-            if (t == ps.t0) {
+            f2* p = chain + s * 96;
+            if (t < ps.t0 + kChains) {
                 p[0] = k.sx[s];
                 p[32] = k.sy[s];
                 p[64] = k.sz[s];
@@ -785,15 +798,22 @@ __device__ __forceinline__ void run_pass(const Pass& ps, int R, const Coef& cf, 
         }
         __syncwarp();
     }
-    // the residents' partial sums
+    // the residents' partial sums: the chains join the first tile's
+    f2* const sums = tot + (ps.t0 & (kChains - 1)) * L::chain;
+#pragma unroll 1
+    for (int t = ps.t0 + 1; t < min(ps.t0 + kChains, ps.t1); ++t) {
+        const f2* other = tot + (t & (kChains - 1)) * L::chain;
+#pragma unroll
+        for (int q = 0; q < 3 * G; ++q) sums[q * 32] = add2(sums[q * 32], other[q * 32]);
+    }
     {
         int q = 0;
 #pragma unroll
         for (int s = 0; s < G; ++s) {
-            const f2* p = tot + (size_t)s * L::NS * 32;
+            const f2* p = sums + s * 96;
             const bool any = ps.t0 < ps.t1;
             const f2 x = any ? p[0] : 0ull, y = any ? p[32] : 0ull, z = any ? p[64] : 0ull;
-            const f2 w = DENS ? p[DENS ? 96 : 0] : 0ull;
+            const f2 w = DENS ? totw[s * TS] : 0ull;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int pos = ps.r0 + (2 * s + h) * 32 + lane;
