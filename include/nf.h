@@ -438,8 +438,10 @@ int nf_timestep(const float *pos, const float *vel, const float *acc, int64_t N,
 /* One leapfrog step in place, all on the device:
  *     vel += acc dt/2;  pos = wrap(pos + vel dt) into [0, box);
  *     acc = nf_forces(pos);  vel += acc dt/2;
- * (nf_forces by the directed kernel at every size, see nf_tuning.)  acc must hold the accelerations at the input positions (from nf_forces or
- * the previous step).  dt is ONE double in device memory: it is read for this
+ * where nf_forces runs in the directed kernel at every size (see nf_tuning), so
+ * that for boxes of the symmetric one acc equals a separate call's to rounding
+ * only.  acc must hold the accelerations at the input positions (from nf_forces
+ * or the previous step).  dt is ONE double in device memory: it is read for this
  * step and, when prm != NULL, overwritten with the next step's dt from
  * Eq. (timestep) at the new state; so a loop of steps needs no host round trip
  * and can be captured in a CUDA graph.  Arguments as nf_forces otherwise. */

@@ -162,19 +162,22 @@ size_t directed_bytes(int64_t N, int64_t C, int R)
 // Which boxes the symmetric pair kernel runs (nf_sym.cu): those of the built-in
 // tuning of the direction with N within these and too large for nf_forces_noalloc,
 // whose fixed scratch cannot hold the partial planes and whose results are
-// nf_forces'.  From 64^3 particles on it is the faster one (pair kernel, clustered:
-// forward 0.89 against 0.99 ms, adjoint 1.59 against 1.80); a smaller box has too few
-// pencils for its warps.  Above, or where a wide stencil has many slots, the planes (18
-// slots of 16 bytes a particle at R = 2, 50 at R = 4) would take over 80 GB.  The time steps stay on the directed kernel: the step size
-// they write is a double made of a few of the FP32 accelerations, read back by the
-// next step, so the last bits of the sums decide a run's trajectory, and a run
-// continued with this version keeps it.
+// nf_forces'.  A smaller box has too few pencils for its warps; which of the larger ones
+// gain is decided by their pencils (sym_box below, box_is_sym in nf_sym.cu: the adjoint of
+// the clustered 64^3 box gains, its forward call does not).  Above, or where a wide stencil
+// has many slots, the planes (18 slots of 16 bytes a particle at R = 2, 50 at R = 4) would
+// take over 80 GB.
+//   The time steps stay on the directed kernel: the step size they write is a double made
+// of a few of the FP32 accelerations and read back by the next step, so the last bits of
+// the sums decide a trajectory, and a step from given positions, velocities and
+// accelerations keeps its bits.  (The accelerations that a run starts from, nf_forces', can
+// be the symmetric kernel's: equal to the directed ones to rounding, not bit for bit.)
 constexpr int64_t kSymMinN = int64_t(1) << 18, kSymMaxN = int64_t(1) << 28;
 constexpr int64_t kSymMaxPlaneBytes = 80000000000;
 // The boxes of a batch share planes of this size (or of its largest box): those that do
 // not fit side by side run in rounds, one after the other on the same planes, so that a
 // batch of many boxes needs little more than its directed rows (300 boxes of 10^6
-// particles: 51 GB; 300 GB with planes for all).
+// particles: 52 GB; 300 GB with planes for all).
 constexpr int64_t kSymRoundPlaneBytes = int64_t(8) << 30;
 // A box whose pencils hold too few sinks at mean occupancy for the symmetric
 // kernel's lanes (fill_needed) is not considered: the choice costs two launches.

@@ -94,7 +94,7 @@ struct CellCoord {
 // runs FP64 at 1/64 of its FP32 rate, so the rule in doubles (cell_coord_fp64)
 // bounds the binning: 3 * 10^7 particles at K / box = 101 / 500 took 1333 us for the
 // cell ids and 1838 us for the first sort pass in doubles, 287 and 670 us this way
-// (and 96 and 461 us with the float pairs of cell_coord before it).
+// (and 96 and 461 us with the float pairs of cell_short before it).
 // Takes 2^-10 <= t < 2^52 for x > 0 (2^-1 <= |t| for x < 0, below which 1 - |t| rounds);
 // the rest, zeros and subnormals go through doubles.  Both give the same bits.
 // Out of line: the sort passes inline only cell_coord's short paths, which keeps their code (24 coordinates per thread) small.

@@ -55,12 +55,13 @@ namespace {
 // whose pencils hold 320 sinks, 45.8, 48.2 and 46.6; 8 warps are slower), adjoint
 // 5 groups at 8 warps 55.0 ms (4: 59.2; 6: 57.3; 3 at 16 warps: 58).  The
 // directed kernel takes 38.7 and 72.9 ms (uniform 256^3: 51.6 and 97.4).
-// What bounds the loop is not the FMA pipe's issue rate but its operands: a packed
-// FMA with three different 64-bit sources (the six sums of a group) takes 3 cycles
-// of the pipe where one with two takes 2, and a shuffle about 2.6.  The bare loop
-// reaches 13 ordered pairs per clock and SM of the 18.3 that 14 operations allow
-// (directed: 10.3 of 11.6).  Unrolling, scalar sums, sums rotated through shared
-// memory and prefetched sources all measured slower.
+// What bounds the loop is not the FMA pipe's issue rate but its operands: run alone in a
+// loop, a packed FMA with three different 64-bit sources (the six sums of a group) took
+// 3.1 cycles a scheduler where one with two took 2.0, and a shuffle held up the FMAs for
+// 2.65.  The bare tile loop reached 13 ordered pairs per clock and SM of the 18.3 that 14
+// operations allow (directed: 10.3 of 11.6).  Unrolling, scalar sums, sums rotated through
+// shared memory and prefetched sources all measured slower.  The registers are full:
+// forward 128, with 24 bytes of spills written and 52 read, adjoint 255, with 68 and 128.
 constexpr int kGroupsFwd = 3, kBlocksFwd = 2;
 constexpr int kGroupsAdj = 5, kBlocksAdj = 1;
 constexpr int kWarps = 8;
