@@ -210,11 +210,16 @@ int sym_box_groups(int64_t N)
 // 938 against 998 with four; adjoint 174 -> 111, 290 -> 234, 373 -> 342, and 602 against
 // 631 with four at 3000 items.
 // With few stages to an item (R = 1) there is less to share: 265000 particles in 19^3
-// cells (6859 items of 4 stages) take 282 us with one warp and 307 with four.
-int coop_warps(int64_t items, int64_t stages, bool adjoint)
+// cells (6859 items of 4 stages) take 282 us with one warp and 307 with four.  Above two
+// waves of full items (`full`: the sinks over a chunk's size, not rounded up per pencil) a
+// uniform box loses: 171672 particles in 15^3 cells (6750 items, all full) take 585 us with
+// one warp and 625 with four, 120000 in 13^3 at R = 3 1041 and 1083, while 131072 in 13^3
+// (6591 items, 5120 full) take 554 and 537.  (Below, some uniform boxes whose full items
+// just fit one wave lose up to 2.5 %, clustered ones of the size gain 1.3 to 1.9 times.)
+int coop_warps(int64_t items, int64_t full, int64_t stages, bool adjoint)
 {
     if (adjoint) return items < 2000 ? 4 : 1;
-    return items < 1000 ? 8 : items < (stages >= 8 * items ? 8000 : 2500) ? 4 : 1;
+    return items < 1000 ? 8 : items < (stages >= 8 * items && full < 5500 ? 8000 : 2500) ? 4 : 1;
 }
 bool same_tuning(const ForceTuning& a, const ForceTuning& b)
 {
@@ -233,8 +238,9 @@ struct Plan {
     int64_t N = 0;       // total particles
     int64_t C = 0;       // total cells
     int64_t max_items = 0;
-    // work items, and their stages in all, if every cell held its box's mean occupancy
-    int64_t mean_items = 0, mean_stages = 0;
+    // work items, full ones of the same sinks, and the items' stages in all, if every cell
+    // held its box's mean occupancy
+    int64_t mean_items = 0, full_items = 0, mean_stages = 0;
     int max_R = 1;
     int max_nseg = 9;
     int nchunks = 0;     // combine chunks
@@ -313,7 +319,7 @@ int make_plan(const nf_box* boxes, int nboxes, bool need_force, int chunk_lanes,
     p->boxes.resize(nboxes);
     int64_t N = 0, C = 0, items = 0, nchunks = 0, units = 0, partials = 0;
     p->any_sym = false;
-    p->mean_items = p->mean_stages = 0;
+    p->mean_items = p->full_items = p->mean_stages = 0;
     int max_R = 1;
     for (int b = 0; b < nboxes; ++b) {
         int rc = make_box(boxes[b], need_force, &p->boxes[b]);
@@ -343,6 +349,7 @@ int make_plan(const nf_box* boxes, int nboxes, bool need_force, int chunk_lanes,
             const int64_t ns = 2 * (int64_t)d.R + 1;
             const int64_t mean = cells * ((ns * d.N / cells + chunk_lanes - 1) / chunk_lanes);
             p->mean_items += mean;
+            p->full_items += ns * d.N / chunk_lanes;
             p->mean_stages += mean * (1 + ns * ns * d.N / cells / 128);
         }
         if (N >= (int64_t(1) << 31)) return fail(NF_ERR_ARG, "total N must be < 2^31");
@@ -572,7 +579,9 @@ int run_forces(const Plan& p, bool adjoint, const ForceTuning& t, const float* p
     const char* sym_name = adjoint ? "symmetric adjoint kernel" : "symmetric force kernel";
     if (p.any_sym) NF_CUDA(sym_force(), sym_name);
     // (with nothing on its list where every box is symmetric)
-    const int coop = builtin_tuning(t, adjoint) && !p.any_sym ? coop_warps(p.mean_items, p.mean_stages, adjoint) : 1;
+    const int coop = builtin_tuning(t, adjoint) && !p.any_sym
+                         ? coop_warps(p.mean_items, p.full_items, p.mean_stages, adjoint)
+                         : 1;
     NF_CUDA(launch_force(adjoint, rho != nullptr, t, coop, boxes, off, rel, gs, items, hdr, partial,
                          pstride, p.max_nseg, s),
             adjoint ? "adjoint kernel" : "force kernel");
