@@ -234,7 +234,7 @@ void nf_get_default_tuning_adjoint(nf_tuning *t);
 /* Workspace for a batch (host array boxes[nboxes]); 0 if the batch is invalid.
  * The boxes share the symmetric kernel's partial sums: 8 GiB of them at most, or
  * what the largest box needs alone, beside the directed kernel's.  Boxes that do
- * not fit side by side run in rounds. */
+ * not fit side by side run in lots. */
 size_t nf_workspace_bytes_batched(const nf_box *boxes, int nboxes);
 
 /* Near-field accelerations of nboxes independent periodic boxes in one pass:

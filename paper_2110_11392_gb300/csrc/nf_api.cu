@@ -175,10 +175,10 @@ size_t directed_bytes(int64_t N, int64_t C, int R)
 constexpr int64_t kSymMinN = int64_t(1) << 18, kSymMaxN = int64_t(1) << 28;
 constexpr int64_t kSymMaxPlaneBytes = 80000000000;
 // The boxes of a batch share planes of this size (or of its largest box): those that do
-// not fit side by side run in rounds, one after the other on the same planes, so that a
+// not fit side by side run in lots, one after the other on the same planes, so that a
 // batch of many boxes needs little more than its directed rows (300 boxes of 10^6
 // particles: 52 GB; 300 GB with planes for all).
-constexpr int64_t kSymRoundPlaneBytes = int64_t(8) << 30;
+constexpr int64_t kSymLotPlaneBytes = int64_t(8) << 30;
 // A box whose pencils hold too few sinks at mean occupancy for the symmetric
 // kernel's lanes (fill_needed) is not considered: the choice costs two launches.
 int sym_box_groups(int64_t N);
@@ -245,11 +245,11 @@ struct Plan {
     int max_nseg = 9;
     int nchunks = 0;     // combine chunks
     bool any_sym = false;  // boxes that may run in the symmetric pair kernel
-    // rounds of the symmetric boxes: consecutive boxes, by their cells and combine chunks
-    struct Round {
+    // lots of the symmetric boxes: consecutive boxes, by their cells and combine chunks
+    struct Lot {
         int c0, c1, chunk0, chunk1;
     };
-    std::vector<Round> rounds;
+    std::vector<Lot> lots;
     SortPlan sp{};
     std::vector<BoxDev> boxes;
     // region offsets (bytes from ws)
@@ -363,28 +363,28 @@ int make_plan(const nf_box* boxes, int nboxes, bool need_force, int chunk_lanes,
     p->max_nseg = (2 * max_R + 1) * (2 * max_R + 1);
     p->nchunks = (int)nchunks;
     if (need_force) {
-        // partial sums in bytes: every particle's row (directed), then the planes of a round's
+        // partial sums in bytes: every particle's row (directed), then the planes of a lot's
         // symmetric boxes; a single box uses one or the other, so both start at the same place
         partials = 16 * (2 * (int64_t)max_R + 1) * N;
         const int64_t first = nboxes == 1 ? 0 : partials;
-        int64_t planes = 0, round_units = 0;
-        p->rounds.assign(1, Plan::Round{0, 0, 0, 0});
+        int64_t planes = 0, lot_units = 0;
+        p->lots.assign(1, Plan::Lot{0, 0, 0, 0});
         for (BoxDev& d : p->boxes) {
-            Plan::Round* r = &p->rounds.back();
+            Plan::Lot* r = &p->lots.back();
             const int cells = d.K * d.K * d.K;
             if (d.sym) {
                 const int64_t size = sym_plane_bytes(d.N, d.R);
-                if (planes > 0 && planes + size > kSymRoundPlaneBytes) {
-                    p->rounds.push_back(Plan::Round{r->c1, r->c1, r->chunk1, r->chunk1});
-                    r = &p->rounds.back();
-                    planes = round_units = 0;
+                if (planes > 0 && planes + size > kSymLotPlaneBytes) {
+                    p->lots.push_back(Plan::Lot{r->c1, r->c1, r->chunk1, r->chunk1});
+                    r = &p->lots.back();
+                    planes = lot_units = 0;
                 }
-                d.round = (int)p->rounds.size() - 1;
+                d.lot = (int)p->lots.size() - 1;
                 d.plane_base = (first + planes) / 4;
                 planes += size;
-                round_units += sym_max_units(d.N, cells, d.R, d.groups);
+                lot_units += sym_max_units(d.N, cells, d.R, d.groups);
                 partials = std::max(partials, first + planes);
-                units = std::max(units, round_units);
+                units = std::max(units, lot_units);
             }
             r->c1 = d.cell_base + cells;
             r->chunk1 = d.chunk_base + (d.N + kCombineChunk - 1) / kCombineChunk;
@@ -554,10 +554,10 @@ int run_forces(const Plan& p, bool adjoint, const ForceTuning& t, const float* p
                            sym_total, gm, hdr, s),
             "pencils");
     int4* items = at<int4>(ws, p.o_items);
-    // the symmetric boxes' work list, round by round (the directed list with the first)
-    auto sym_units = [&](int round) {
-        const Plan::Round& r = p.rounds[round];
-        return launch_sym_units(adjoint, boxes, p.nboxes, round, r.c0, round == 0 ? (int)p.C : r.c1, off, dims, sym,
+    // the symmetric boxes' work list, lot by lot (the directed list with the first)
+    auto sym_units = [&](int lot) {
+        const Plan::Lot& r = p.lots[lot];
+        return launch_sym_units(adjoint, boxes, p.nboxes, lot, r.c0, lot == 0 ? (int)p.C : r.c1, off, dims, sym,
                                 sym_total, units, chunks, bucket_of, bucket_count, items, hdr, s);
     };
     if (p.any_sym) {
@@ -586,18 +586,18 @@ int run_forces(const Plan& p, bool adjoint, const ForceTuning& t, const float* p
                          pstride, p.max_nseg, s),
             adjoint ? "adjoint kernel" : "force kernel");
     double* chunk_sums = net ? at<double>(ws, p.o_chunk_sums) : nullptr;
-    auto combine = [&](const Plan::Round& r) {
+    auto combine = [&](const Plan::Lot& r) {
         return launch_combine(adjoint, boxes, p.nboxes, r.chunk0, r.chunk1 - r.chunk0, partial, pstride, perm, out,
                               rho, chunk_sums, s);
     };
-    // each round's planes are combined before the next one writes them
-    for (size_t q = 1; q < p.rounds.size(); ++q) {
-        NF_CUDA(combine(p.rounds[q - 1]), "combine");
+    // each lot's planes are combined before the next one writes them
+    for (size_t q = 1; q < p.lots.size(); ++q) {
+        NF_CUDA(combine(p.lots[q - 1]), "combine");
         NF_CUDA(sym_units((int)q), "work units");
         NF_CUDA(sym_force(), sym_name);
     }
     NF_CUDA(prof_mark(3, s), "profile");
-    NF_CUDA(combine(p.rounds.back()), "combine");
+    NF_CUDA(combine(p.lots.back()), "combine");
     if (net) NF_CUDA(launch_net(boxes, p.nboxes, chunk_sums, net, s), "net force");
     NF_CUDA(prof_mark(4, s), "profile");
     if (g_profile_on) ++g_prof_count;

@@ -56,8 +56,8 @@ struct BoxDev {
     float kl_pow2;
     // K / box as a float pair, or 0 outside FP32's middle range
     float kl_hi, kl_lo;
-    // pass over the batch in which a symmetric box runs (make_plan)
-    int round;
+    // lot of a batch in which a symmetric box runs (make_plan)
+    int lot;
     int pad;
     // 1: the top-hat term runs only in the pair-kernel stages where some pair
     // is closer than b (small b); 0: it is fused into every stage that can hold one
@@ -302,10 +302,10 @@ long long sym_max_units(long long N, long long C, int R, int groups);
 // total: [3 nboxes], the boxes' costs, the costs of their dear pencils (written here), and
 // the directed kernel's lane pairs.
 // Clears .sym of the boxes that run better directed; writes both lists (bucket_count holds
-// the other boxes' chunks).  Round 0 takes all cells [0, c1) and writes the directed list
-// whole; a later one, its boxes' cells [c0, c1).  units and ctl (cleared here after round
-// 0) hold one round's list.
-cudaError_t launch_sym_units(bool adjoint, BoxDev* boxes, int nboxes, int round, int c0, int c1, const int* cell_off,
+// the other boxes' chunks).  Lot 0 takes all cells [0, c1) and writes the directed list
+// whole; a later one, its boxes' cells [c0, c1).  units and ctl (cleared here after lot
+// 0) hold one lot's list.
+cudaError_t launch_sym_units(bool adjoint, BoxDev* boxes, int nboxes, int lot, int c0, int c1, const int* cell_off,
                              const int2* dims, SymCtl* ctl, unsigned long long* total, int4* units,
                              const int* chunks, const unsigned char* bucket_of, unsigned* bucket_count, int4* items,
                              WsHeader* hdr, cudaStream_t s);

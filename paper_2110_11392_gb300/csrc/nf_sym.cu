@@ -174,8 +174,8 @@ __device__ __forceinline__ bool box_is_sym(const BoxDev* boxes, int nboxes, cons
     return (double)total[nboxes + b] <= dear_share(adjoint) * cost && fill >= fill_needed(boxes[b].N, adjoint);
 }
 
-// Counts the units of the round's boxes and, in round 0, the chunks of all that turn out directed.
-__global__ void k_sym_count(const BoxDev* __restrict__ boxes, int nboxes, int round, int c0, int c1,
+// Counts the units of the lot's boxes and, in lot 0, the chunks of all that turn out directed.
+__global__ void k_sym_count(const BoxDev* __restrict__ boxes, int nboxes, int lot, int c0, int c1,
                             const int* __restrict__ off,
                             const int2* __restrict__ dims, const unsigned long long* __restrict__ total, int GM,
                             int warps, bool adjoint, const int* __restrict__ chunks,
@@ -191,14 +191,14 @@ __global__ void k_sym_count(const BoxDev* __restrict__ boxes, int nboxes, int ro
         if (c < c1) {
             const int b = find_box_by_cell(boxes, nboxes, c);
             if (nboxes == 1 ? one_sym : box_is_sym(boxes, nboxes, total, b, adjoint)) {
-                if (boxes[b].round == round) {
+                if (boxes[b].lot == lot) {
                     const int2 d = dims[c];
                     const UnitCount u =
                         count_units(d.x, d.y, off[c + 1] - off[c], boxes[b].groups, GM, (double)total[b] / warps);
                     n = u.units;
                     if (n) bk = u.bucket;
                 }
-            } else if (round == 0 && boxes[b].sym) {  // a candidate: its chunks are not counted yet
+            } else if (lot == 0 && boxes[b].sym) {  // a candidate: its chunks are not counted yet
                 n = chunks[c];
                 if (n) bk = kBuckets + (int)bucket_of[c];
             }
@@ -210,7 +210,7 @@ __global__ void k_sym_count(const BoxDev* __restrict__ boxes, int nboxes, int ro
     }
 }
 
-// Exclusive scans of both lists' buckets (round 0; later the units' alone, in kBuckets
+// Exclusive scans of both lists' buckets (lot 0; later the units' alone, in kBuckets
 // threads); the boxes' kernels for good.
 __global__ void k_sym_scan(BoxDev* boxes, int nboxes, const unsigned long long* __restrict__ total, bool adjoint,
                            SymCtl* ctl, unsigned* dir_count, WsHeader* hdr)
@@ -239,9 +239,9 @@ __global__ void k_sym_scan(BoxDev* boxes, int nboxes, const unsigned long long* 
 // Unit types (item .w)
 constexpr int kUnitSym = 0, kUnitSinks = 1, kUnitSources = 2;
 
-// Writes both lists bucket by bucket (as k_items): the round's symmetric units and, in
-// round 0, the directed items of the other boxes.
-__global__ void k_sym_units(const BoxDev* __restrict__ boxes, int nboxes, int round, int c0, int c1,
+// Writes both lists bucket by bucket (as k_items): the lot's symmetric units and, in
+// lot 0, the directed items of the other boxes.
+__global__ void k_sym_units(const BoxDev* __restrict__ boxes, int nboxes, int lot, int c0, int c1,
                             const int* __restrict__ off,
                             const int2* __restrict__ dims, const unsigned long long* __restrict__ total, int GM,
                             int warps, const int* __restrict__ chunks, const unsigned char* __restrict__ bucket_of,
@@ -256,14 +256,14 @@ __global__ void k_sym_units(const BoxDev* __restrict__ boxes, int nboxes, int ro
         if (c < c1) {
             b = find_box_by_cell(boxes, nboxes, c);
             if (boxes[b].sym) {
-                if (boxes[b].round == round) {
+                if (boxes[b].lot == lot) {
                     const int2 d = dims[c];
                     groups = boxes[b].groups;
                     u = count_units(d.x, d.y, off[c + 1] - off[c], groups, GM, (double)total[b] / warps);
                     n = u.units;
                     if (n) bk = u.bucket;
                 }
-            } else if (round == 0) {
+            } else if (lot == 0) {
                 n = chunks[c];
                 if (n) bk = kBuckets + (int)bucket_of[c];
             }
@@ -1042,23 +1042,23 @@ long long sym_max_units(long long N, long long C, int R, int groups)
     return C * (2 * (long long)groups + 2) + (ns * groups + nb) * (N / 64 + 1);
 }
 
-cudaError_t launch_sym_units(bool adjoint, BoxDev* boxes, int nboxes, int round, int c0, int c1, const int* cell_off,
+cudaError_t launch_sym_units(bool adjoint, BoxDev* boxes, int nboxes, int lot, int c0, int c1, const int* cell_off,
                              const int2* dims, SymCtl* ctl, unsigned long long* total, int4* units,
                              const int* chunks, const unsigned char* bucket_of, unsigned* bucket_count, int4* items,
                              WsHeader* hdr, cudaStream_t s)
 {
     const int grid = grid_for(c1 - c0, 256), warps = sym_warps(adjoint), GM = sym_groups_max(adjoint);
-    if (round == 0) {
+    if (lot == 0) {
         k_sym_dear<<<grid, 256, 0, s>>>(boxes, nboxes, c1, cell_off, dims, total, GM, warps);
         count_launches(1);
     } else {
         const cudaError_t e = cudaMemsetAsync(ctl, 0, sizeof(SymCtl), s);
         if (e != cudaSuccess) return e;
     }
-    k_sym_count<<<grid, 256, 0, s>>>(boxes, nboxes, round, c0, c1, cell_off, dims, total, GM, warps, adjoint, chunks,
+    k_sym_count<<<grid, 256, 0, s>>>(boxes, nboxes, lot, c0, c1, cell_off, dims, total, GM, warps, adjoint, chunks,
                                      bucket_of, ctl->bucket, bucket_count);
-    k_sym_scan<<<1, (round == 0 ? 2 : 1) * kBuckets, 0, s>>>(boxes, nboxes, total, adjoint, ctl, bucket_count, hdr);
-    k_sym_units<<<grid, 256, 0, s>>>(boxes, nboxes, round, c0, c1, cell_off, dims, total, GM, warps, chunks,
+    k_sym_scan<<<1, (lot == 0 ? 2 : 1) * kBuckets, 0, s>>>(boxes, nboxes, total, adjoint, ctl, bucket_count, hdr);
+    k_sym_units<<<grid, 256, 0, s>>>(boxes, nboxes, lot, c0, c1, cell_off, dims, total, GM, warps, chunks,
                                      bucket_of, ctl->bucket, bucket_count, units, items);
     count_launches(3);
     return cudaGetLastError();

@@ -1,4 +1,4 @@
-"""A batch whose symmetric boxes do not fit side by side in the shared partial sums runs in rounds: bit for bit the
+"""A batch whose symmetric boxes do not fit side by side in the shared partial sums runs in lots: bit for bit the
 single calls, forward (with the net force), adjoint and replayed from a graph."""
 import numpy as np
 import pytest
@@ -10,11 +10,11 @@ from _helpers import to_dev
 pytestmark = pytest.mark.gpu
 
 
-def test_rounds_equal_single_calls():
+def test_lots_equal_single_calls():
     import torch
     import paper_2110_11392_gb300 as nf
     from paper_2110_11392_gb300 import _lib
-    # 2.5 GB of planes each for the large boxes (113 slots): three fit in 8 GiB, so there are two rounds, with
+    # 2.5 GB of planes each for the large boxes (113 slots): three fit in 8 GiB, so there are two lots, with
     # directed boxes in both
     parts = [(1400003, 30, 4), (5000, 9, 2), (1400001, 30, 4), (1399999, 30, 4), (1400007, 30, 4), (4001, 9, 4)]
     pos = [uniform_positions(N, q + 1) for q, (N, _, _) in enumerate(parts)]

@@ -18,7 +18,7 @@ def directed_bytes(N, K, R, chunk=32):
 def test_batch_of_many_boxes():
     n, N, K, R = 300, 10 ** 6, 25, 2
     need = _lib.nf_workspace_bytes_batched(batch(n, N, K, R))
-    # 5 % for the tables per cell, the sort's counts and the work units of one round
+    # 5 % for the tables per cell, the sort's counts and the work units of one lot
     assert 0 < need <= 1.05 * n * directed_bytes(N, K, R) + (8 << 30) + (1 << 30), need
 
 
